@@ -2487,33 +2487,52 @@ __global__ void __launch_bounds__(128, 4) k_epf(const __grid_constant__ FilterAr
 //   k_epf_work  persistent one-warp CTAs taking 2 listed blocks at a time
 //               (a group; the warps claim groups from a per-request counter):
 //               per block a window of mirrored samples and packed guide
-//               bytes (6.5, J.2.2), then per horizontal offset ox
-//               step 1  the horizontal 4-sums H_o of the 10 rows the block's
-//                       3x4 patches touch (block rows -1..8) for the 7
-//                       vertical offsets, as 16-bit values, one lane per
-//                       (block, row) walking the 7 offsets with its own
-//                       guide bytes in registers;
-//               step 2  one lane per half column (4 rows) of a block: the
-//                       sliding vertical 3-sums (the patch SADs) of the 7
-//                       vertical offsets, a warp vote on which offsets give
-//                       some pixel a weight above the J.2.4 cut-off, and for
-//                       those only the weights and the J.2.5 sums.
+//               bytes (6.5, J.2.2), the bytes then regrouped as planar words
+//               (4 neighbouring columns of one channel, one word per start
+//               column), so that one byte-SAD instruction takes 4 columns of
+//               a patch row.  A lane holds half a column of a block (4
+//               pixels): per horizontal offset it loads the 12 x 3 neighbour
+//               words once, forms the 6 patch-row sums of each of the 7
+//               vertical offsets (3 chained SADs each), adds 3 rows per
+//               pixel, and keeps the 28 patch SADs in registers for the warp
+//               votes (any of the 7 offsets live, then which) and for the
+//               live ones the weights and the J.2.5 sums.
 //               Weights, cut-off and summation order are those of k_epf, so
 //               the two kernels give the same bits (an offset skipped by
 //               the vote would add exactly zero).  Warps synchronise only
 //               within themselves: a CTA never waits on another warp.
+//
+// Bound by the integer pipe (half rate: 126 SADs, 28 three-way adds and 17
+// minima per lane and horizontal offset) and, at 16 warps per SM, by the
+// latency of the window loads: ALU pipe 64% busy at 2048^2.  Against the
+// earlier form (one SAD per pixel, packed horizontal 4-sums through shared
+// memory, 16-bit loads back for the vertical sums: 13 instructions per pixel
+// and offset instead of 7.5) the whole step at 4096^2 takes 0.645 ms instead
+// of 0.717 (this kernel 0.307 -> 0.235), at 3001x2003 with most offsets live
+// 0.425 instead of 0.460.  A lane per whole column (8 pixels, 4 blocks per
+// warp) has 12% fewer instructions but only 8 warps per SM and takes longer
+// (0.692 and 0.555 ms for the same steps).
 // ---------------------------------------------------------------------------
 constexpr int kLG = 2;                            // blocks per warp and round (the lane
-                                                  // layout of step 2 assumes 2)
+                                                  // layout of the sums assumes 2)
 constexpr int kLGH = 16, kLGW = 18, kLGS = 19;    // guide window, origin (-4, -4) of the block
+constexpr int kLWC = 15, kLWS = 20;               // planar guide words: start columns, words per
+                                                  // column (16 rows, 16-byte multiples)
+constexpr int kLWB = 912;                         // words per block (>= 3 kLWC kLWS, = 16 mod 32)
 constexpr int kLFH = 14, kLFW = 15, kLFS = 16;    // sample window, origin (-3, -3); row stride
 constexpr int kLFC = kLFH * kLFS;                 // floats per channel
 constexpr int kLFB = 688;                         // floats per block (>= 3 kLFC, = 16 mod 32)
 // Column of sample (row fr, column fc) in its row: rows 4 apart (the two
-// half-column lane groups of step 2) swap their 8-column halves, so that the
-// groups read different banks.
+// half-column lane groups) swap their 8-column halves, so that the groups
+// read different banks.
 __device__ __forceinline__ int lf_col(int fr, int fc) { return fc ^ (((fr >> 2) & 1) << 3); }
-constexpr int kLHR = 10;                          // rows of horizontal sums per block
+
+// acc + sum over the four bytes of |a - b|.
+__device__ __forceinline__ uint32_t sad4(uint32_t a, uint32_t b, uint32_t acc) {
+  uint32_t d;
+  asm("vabsdiff4.u32.u32.u32.add %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(acc));
+  return d;
+}
 
 // The groups of one image's list (total listed blocks) a warp takes: g0,
 // g0 + gs, ... or, with next (a zeroed counter), the ones it claims there one
@@ -2522,13 +2541,13 @@ template <bool kClamp>
 __device__ __forceinline__ void epf_work_groups(const FilterArgs& a, const int* __restrict__ list,
                                                 int total, int g0, int gs,
                                                 unsigned* next = nullptr) {
-  __shared__ uint32_t G[kLG][kLGH][kLGS];
+  __shared__ __align__(16) uint32_t W[kLG][kLWB];
   __shared__ float F[kLG][kLFB];
-  __shared__ __align__(16) uint16_t Hb[kLG][7][kLHR][8];
+  static_assert(kLGH * kLGS <= kLWB && 3 * kLWC * kLWS <= kLWB, "window sizes");
   const int lane = threadIdx.x;
   const int C = 0x3F800000;
   const int T16 = static_cast<int>((a.wmin_bits + 0xFFFFu) & 0xFFFF0000u);
-  // step 2: lane = (block sk, rows 4 hh .. 4 hh + 3, column cx)
+  // lane = (block sk, rows 4 hh .. 4 hh + 3, column cx)
   const int sk = lane >> 4, hh = (lane >> 3) & 1, cx = lane & 7, r0 = 4 * hh;
   int grp = g0;
   if (next) {
@@ -2570,7 +2589,7 @@ __device__ __forceinline__ void epf_work_groups(const FilterArgs& a, const int* 
           const float sc = fminf(fmaxf(guide_scaled(a.sp, c, wv[q][c]), 0.f), 255.f);
           g |= static_cast<uint32_t>(sc) << (8 * c);
         }
-        G[k][ly][lx] = g;
+        W[k][ly * kLGS + lx] = g;
         if (ly >= 1 && ly <= kLFH && lx >= 1 && lx <= kLFW) {
 #pragma unroll
           for (int c = 0; c < 3; ++c)
@@ -2578,8 +2597,30 @@ __device__ __forceinline__ void epf_work_groups(const FilterArgs& a, const int* 
         }
       }
     }
+    __syncwarp();
+    // ---- planar guide words: lane = (block, window row); the word of channel
+    // c at start column s holds that channel's bytes of columns s .. s + 3 ----
+    {
+      const int row = lane & 15;
+      uint32_t* Wk = &W[lane >> 4][0];
+      uint32_t g[kLGW];
+#pragma unroll
+      for (int i = 0; i < kLGW; ++i) g[i] = Wk[row * kLGS + i];
+      __syncwarp();
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        uint32_t w = __byte_perm(__byte_perm(g[0], g[1], c | (4 + c) << 4),
+                                 __byte_perm(g[2], g[3], c | (4 + c) << 4), 0x5410);
+        Wk[c * kLWC * kLWS + row] = w;
+#pragma unroll
+        for (int s = 1; s < kLWC; ++s) {
+          w = __byte_perm(w, g[s + 3], 0x0321 | (4 + c) << 12);
+          Wk[(c * kLWC + s) * kLWS + row] = w;
+        }
+      }
+    }
 
-    // ---- this lane's half column (step 2) --------------------------------
+    // ---- this lane's half column -----------------------------------------
     const bool strip = sk < nb;
     const int sb0 = strip ? __ldg(list + kLG * grp + sk) : 0;
     const int sby = sb0 / a.bw, sbx = sb0 - sby * a.bw;
@@ -2595,85 +2636,57 @@ __device__ __forceinline__ void epf_work_groups(const FilterArgs& a, const int* 
     float2 ax[2], ay[2], ab[2], ws[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) ax[q] = ay[q] = ab[q] = ws[q] = make_float2(0.f, 0.f);
-    // step 1: 140 units (block, row, vertical offset) over the 32 lanes in 5
-    // rounds.  Lanes 0..19 = (block, row) take the offsets oy = -3 .. 1 of
-    // their row (rounds 0..4, own guide bytes loaded once); lanes 20..31
-    // take the (block, row) pairs 0..11 and then 12..19 for oy = 2 and 3
-    // (rounds 0, 1 and 2, 3, own bytes loaded again at round 2).
-    const bool grpA = lane < 2 * kLHR;
-    const int pa = grpA ? lane : lane - 2 * kLHR;       // (block, row) pair of rounds 0, 1
-    const int pb = grpA ? lane : lane - 2 * kLHR + 12;  // ... of rounds 2, 3
-    // the word offsets in G of the rows of those pairs, the 16-bit offsets
-    // in Hb of their sums, and whether the pairs exist (none depends on ox)
-    const int ka = pa >= kLHR ? 1 : 0, ja = pa - kLHR * ka;
-    const int kb = pb >= kLHR ? 1 : 0, jb = pb - kLHR * kb;
-    const int goa = (ka * kLGH + ja) * kLGS, gob = (kb * kLGH + jb) * kLGS;
-    const int hoa = (ka * 7 * kLHR + ja) * 8, hob = (kb * 7 * kLHR + jb) * 8;
-    const bool ona = ka < nb, onb = kb < nb && (grpA || pb < 2 * kLHR);
-    bool dense = false;     // step 2: every offset of the last ox was live
     __syncwarp();
+    // the lane's own words: columns cx - 1 .. cx + 2 of block rows r0 - 1 .. r0 + 4
+    const uint32_t* Wl = &W[sk][cx * kLWS + r0];
+    uint32_t own[3][6];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int j = 0; j < 6; ++j) own[c][j] = Wl[(c * kLWC + 3) * kLWS + 3 + j];
 
 #pragma unroll 1
     for (int g = 0; g < 8; ++g) {
       const int ox = g - 3;
-      // ---- step 1 --------------------------------------------------------------
-      {
-        uint32_t own[11];
-        const uint32_t* G0 = &G[0][0][0];
+      // ---- the patch SADs of the lane's 4 pixels for the 7 vertical offsets:
+      // the rows' 4-sums over the three channels, then 3 rows each -----------
+      uint32_t nb4[3][12];   // the neighbour words of window rows r0 .. r0 + 11
 #pragma unroll
-        for (int t = 0; t < 5; ++t) {
-          const int go = t < 2 ? goa : gob, ho = t < 2 ? hoa : hob;   // this round's pair
-          const int oi = grpA ? t : 5 + (t & 1);
-          const bool on = t < 2 ? ona : (onb && (grpA || t < 4));
-          if (t == 0 || t == 2) {
+      for (int c = 0; c < 3; ++c)
 #pragma unroll
-            for (int i = 0; i < 11; ++i) own[i] = on ? G0[go + 3 * kLGS + 3 + i] : 0u;
-          }
-          if (on) {
-            const uint32_t* nbp = G0 + go + oi * kLGS + 3 + ox;
-            uint32_t d[11];   // sum over the 3 channel bytes of |own - neighbour|
-#pragma unroll
-            for (int i = 0; i < 11; ++i) d[i] = __vsadu4(own[i], nbp[i]);
-            *reinterpret_cast<uint4*>(&Hb[0][0][0][0] + ho + oi * kLHR * 8) = hsum4_packed(d);
-          }
+        for (int j = 0; j < 12; j += 4) {
+          const uint4 v = *reinterpret_cast<const uint4*>(Wl + (c * kLWC + g) * kLWS + j);
+          nb4[c][j] = v.x; nb4[c][j + 1] = v.y; nb4[c][j + 2] = v.z; nb4[c][j + 3] = v.w;
         }
-      }
-      __syncwarp();
-
-      // ---- step 2 ----------------------------------------------------------
-      // the patch SADs of the lane's 4 pixels for the 7 offsets, and which
-      // offsets give some pixel of the warp a weight above the cut-off
-      int sad[7][4];
+      int sad[7][4], smin[7];
 #pragma unroll
       for (int oi = 0; oi < 7; ++oi) {
-        int hv[6];
+        uint32_t h[6];
 #pragma unroll
-        for (int jj = 0; jj < 6; ++jj) hv[jj] = strip ? Hb[sk][oi][r0 + jj][cx] : 0;
-        int v = hv[0] + hv[1] + hv[2];
+        for (int j = 0; j < 6; ++j)
+          h[j] = sad4(own[2][j], nb4[2][j + oi],
+                      sad4(own[1][j], nb4[1][j + oi], sad4(own[0][j], nb4[0][j + oi], 0u)));
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          if (r > 0) v += hv[r + 2] - hv[r - 1];
-          sad[oi][r] = v;
-        }
+        for (int r = 0; r < 4; ++r) sad[oi][r] = static_cast<int>(h[r] + h[r + 1] + h[r + 2]);
+        smin[oi] = min(min(sad[oi][0], sad[oi][1]), min(sad[oi][2], sad[oi][3]));
+        // Weight() clamps sad at 507, which matters only in the kClamp variant
+        if (kClamp) smin[oi] = min(smin[oi], 507);
       }
+
+      // ---- J.2.4 weights and J.2.5 sums --------------------------------------
       // An offset none of whose weights passes the cut-off adds exactly zero
-      // to the J.2.5 sums (partial sums start at +0 and never become -0), so
-      // skipping it leaves every result bit unchanged.  Once a horizontal
-      // offset has all 7 offsets live, the group stops testing (computing a
-      // zero weight is as exact as skipping it).
-      unsigned live = 0x7Fu;
-      if (!dense) {
-        live = 0;
+      // to the sums (partial sums start at +0 and never become -0), so skipping
+      // it leaves every result bit unchanged: first the 7 vertical offsets at
+      // once, then each of them.
+      int all = smin[0];
 #pragma unroll
-        for (int oi = 0; oi < 7; ++oi) {
-          const int smin = min(min(sad[oi][0], sad[oi][1]), min(sad[oi][2], sad[oi][3]));
-          // Weight() clamps sad at 507, which matters only in the kClamp variant
-          live |= static_cast<unsigned>((kClamp ? min(smin, 507) : smin) <= vmax) << oi;
-        }
-        live = __reduce_or_sync(0xFFFFFFFFu, live);
-        dense = live == 0x7Fu;
-      }
-      if (live && strip) {
+      for (int oi = 1; oi < 7; ++oi) all = min(all, smin[oi]);
+      if (!__any_sync(0xFFFFFFFFu, all <= vmax)) continue;
+      unsigned live = 0;
+#pragma unroll
+      for (int oi = 0; oi < 7; ++oi) live |= static_cast<unsigned>(smin[oi] <= vmax) << oi;
+      live = __reduce_or_sync(0xFFFFFFFFu, live);
+      {
         const float* Fk = &F[sk][0];
         const int col = cx + ox + 3;
         float sx[10], sy[10], sb[10];
@@ -2712,7 +2725,6 @@ __device__ __forceinline__ void epf_work_groups(const FilterArgs& a, const int* 
           }
         }
       }
-      __syncwarp();
     }
 
     if (strip) {
@@ -2731,13 +2743,13 @@ __device__ __forceinline__ void epf_work_groups(const FilterArgs& a, const int* 
         }
       }
     }
-    __syncwarp();   // the next group's windows overwrite G and F
+    __syncwarp();   // the next group's windows overwrite W and F
     grp = next ? static_cast<int>(__shfl_sync(0xFFFFFFFFu, claim, 0)) : grp + gs;
   }
 }
 
 template <bool kClamp>
-__global__ void __launch_bounds__(32, 20) k_epf_work(const __grid_constant__ FilterArgs a,
+__global__ void __launch_bounds__(32, 16) k_epf_work(const __grid_constant__ FilterArgs a,
                                                      const int* __restrict__ list,
                                                      const unsigned* __restrict__ count,
                                                      unsigned* next) {
@@ -2756,7 +2768,7 @@ __global__ void __launch_bounds__(32, 20) k_epf_work(const __grid_constant__ Fil
 // block is read where it is (warp-uniform loads through L1), so that the
 // shared memory of a warp is that of k_epf_work and as many warps fit.
 template <bool kClamp>
-__global__ void __launch_bounds__(32, 20) k_epf_work_batch(const FilterArgs* __restrict__ args,
+__global__ void __launch_bounds__(32, 16) k_epf_work_batch(const FilterArgs* __restrict__ args,
                                                            const unsigned* __restrict__ counts,
                                                            int nimg, unsigned* next) {
   const unsigned full = 0xFFFFFFFFu;
