@@ -379,6 +379,22 @@ jxlr_status acquire_slot(jxl_recon_ctx* ctx, size_t need, uint64_t pixels, Slot*
   return JXLR_OK;
 }
 
+// acquire_slot() for a request with the EPF: its arena has room for the J.2.2
+// guide bytes behind `need` when the request with them fits under the HBM cap
+// and on the device (*plane), else the request runs without that plane (the
+// J.2 kernel then forms the bytes from the samples), so that it needs no more
+// memory than the filter itself.
+jxlr_status acquire_epf_slot(jxl_recon_ctx* ctx, size_t need, size_t plane_bytes, uint64_t pixels,
+                             Slot** out, bool* plane) {
+  *plane = plane_bytes != 0;
+  jxlr_status st = acquire_slot(ctx, need + plane_bytes, pixels, out);
+  if (st == JXLR_ENOMEM && *plane) {
+    *plane = false;
+    st = acquire_slot(ctx, need, pixels, out);
+  }
+  return st;
+}
+
 struct Carve {
   char* base;
   size_t off = 0;
@@ -438,6 +454,7 @@ static int launch_epf_chain(Slot* slot, const FilterArgs& fa, float* eo, const E
   e.epf_out = eo;
   e.ors = wp;
   e.ops = wp * hp;
+  e.guide = sink.guide;
   mark(slot, 5);
   launch_epf_work(e, sink.list, sink.count, sink.count + 1, s);   // status words 4, 5
   mark(slot, 6);
@@ -545,11 +562,15 @@ extern "C" jxlr_status jxl_recon_submit(jxl_recon_ctx* ctx, const jxl_recon_coef
   const size_t out_bytes = out->row_stride_bytes * (ys - 1) + px_bytes * xs;
   if (!out->on_device) add(out_bytes);
   need = align_up(need, 256);
+  const size_t plane_bytes = fp->epf ? align_up(3 * 64 * nblk, 256) : 0;   // J.2.2 guide bytes
 
   std::lock_guard<std::mutex> lock(ctx->mu);
   CK(cudaSetDevice(ctx->device));
   Slot* slot = nullptr;
-  jxlr_status st = acquire_slot(ctx, need, static_cast<uint64_t>(xs) * static_cast<uint64_t>(ys), &slot);
+  bool plane = false;
+  jxlr_status st = acquire_epf_slot(ctx, need, plane_bytes,
+                                    static_cast<uint64_t>(xs) * static_cast<uint64_t>(ys), &slot,
+                                    &plane);
   if (st != JXLR_OK) return st;
   slot->timed = ctx->timing;
   slot->epf_marked = false;
@@ -670,6 +691,7 @@ extern "C" jxlr_status jxl_recon_submit(jxl_recon_ctx* ctx, const jxl_recon_coef
       sink.pass = eo;
       sink.prs = wp;
       sink.pps = static_cast<size_t>(wp) * hp;
+      if (plane) sink.guide = reinterpret_cast<uint8_t*>(slot->arena + need);
     }
     ra.write_xyb = 1;
     ra.xyb = xyb;
@@ -735,10 +757,14 @@ extern "C" jxlr_status jxl_recon_submit_xyb(jxl_recon_ctx* ctx, const float* xyb
     need += align_up(sizeof(int) * static_cast<size_t>(bw) * bh, 256);
   }
   if (fp->noise) need += align_up(sizeof(float) * 3 * static_cast<size_t>(xs) * ys, 256);
+  const size_t plane_bytes = fp->epf ? align_up(size_t(3) * 64 * bw * bh, 256) : 0;
   std::lock_guard<std::mutex> lock(ctx->mu);
   CK(cudaSetDevice(ctx->device));
   Slot* slot = nullptr;
-  jxlr_status st = acquire_slot(ctx, need, static_cast<uint64_t>(xs) * static_cast<uint64_t>(ys), &slot);
+  bool plane = false;
+  jxlr_status st = acquire_epf_slot(ctx, need, plane_bytes,
+                                    static_cast<uint64_t>(xs) * static_cast<uint64_t>(ys), &slot,
+                                    &plane);
   if (st != JXLR_OK) return st;
   slot->timed = ctx->timing;
   slot->epf_marked = false;
@@ -766,6 +792,7 @@ extern "C" jxlr_status jxl_recon_submit_xyb(jxl_recon_ctx* ctx, const float* xyb
     sink.pass = eo;
     sink.prs = static_cast<size_t>(8) * bw;
     sink.pps = static_cast<size_t>(64) * bw * bh;
+    if (plane) sink.guide = reinterpret_cast<uint8_t*>(slot->arena + need);
     SigmaArgs sa;
     std::memset(&sa, 0, sizeof(sa));
     sa.xyb = xyb;

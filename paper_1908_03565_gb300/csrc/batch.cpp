@@ -48,6 +48,7 @@ struct jxl_recon_batch {
                                    // (ne + 1 words, zeroed per launch)
   int ne = 0, etotal = 0;
   bool clamp = false;
+  bool plane = false;              // the sigma pass stores the J.2.2 guide bytes
   FilterArgs* d_fargs = nullptr;   // Gaborish / colour of every filtered image
   int* d_fprefix = nullptr;
   int nf = 0, ftotal = 0;
@@ -77,8 +78,8 @@ void enqueue(const jxl_recon_batch* b, const int* grid, cudaStream_t s) {
   if (b->ne) cudaMemsetAsync(b->d_counts, 0, sizeof(unsigned) * (b->ne + 1), s);
   if (b->rtotal) launch_recon_batch(b->d_rargs, b->d_ritem, b->rtotal, grid[0], s);
   if (b->ne)
-    launch_epf_work_batch(b->d_eargs, b->d_counts, b->ne, b->clamp, grid[1], b->d_counts + b->ne,
-                          s);
+    launch_epf_work_batch(b->d_eargs, b->d_counts, b->ne, b->clamp, b->plane, grid[1],
+                          b->d_counts + b->ne, s);
   if (b->ftotal) {
     if (b->use_tma)
       launch_filter_batch_tma(b->d_fargs, b->d_fprefix, b->d_maps, b->nf, b->ftotal, grid[2],
@@ -145,7 +146,8 @@ void launch_kind(jxl_recon_batch* b, int k, int g, bool tma) {
     launch_recon_batch(b->d_rargs, b->d_ritem, b->rtotal, g, b->cap);
   } else if (k == 1) {
     cudaMemsetAsync(b->d_counts + b->ne, 0, sizeof(unsigned), b->cap);
-    launch_epf_work_batch(b->d_eargs, b->d_counts, b->ne, b->clamp, g, b->d_counts + b->ne, b->cap);
+    launch_epf_work_batch(b->d_eargs, b->d_counts, b->ne, b->clamp, b->plane, g,
+                          b->d_counts + b->ne, b->cap);
   } else if (tma) {
     launch_filter_batch_tma(b->d_fargs, b->d_fprefix, b->d_maps, b->nf, b->ftotal, g, b->d_err,
                             b->cap);
@@ -372,7 +374,21 @@ extern "C" jxlr_status jxl_recon_batch_create(jxl_recon_ctx* ctx, const jxl_reco
   bool tma = !fa.empty() && !(flags & JXLR_BATCH_PLAIN_LOADS);
   const size_t o_tm = take(sizeof(Map) * fa.size()), o_er = take(sizeof(unsigned));
   const size_t o_sc = take(scratch);
-  cudaError_t e = cudaMalloc(&b->dmem, up(off, 256));
+  // the guide bytes of the images with the EPF behind everything else, when
+  // the device has room for them (else J.2 forms them from the samples)
+  const size_t bytes = up(off, 256);
+  std::vector<size_t> guide_off;
+  size_t guide = 0;
+  for (const FilterArgs& f : ea) {
+    guide_off.push_back(guide);
+    guide += up(3 * f.ops, 256);
+  }
+  cudaError_t e = cudaMalloc(&b->dmem, bytes + guide);
+  b->plane = e == cudaSuccess && guide != 0;
+  if (e != cudaSuccess && guide) {
+    cudaGetLastError();
+    e = cudaMalloc(&b->dmem, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     jxl_recon_batch_destroy(b);
@@ -396,6 +412,8 @@ extern "C" jxlr_status jxl_recon_batch_create(jxl_recon_ctx* ctx, const jxl_reco
     r.epf.pass = eo[eimg[j]];
     r.epf.prs = size_t(r.wp);
     r.epf.pps = size_t(r.wp) * r.hp;
+    if (b->plane) r.epf.guide = reinterpret_cast<uint8_t*>(base + bytes + guide_off[j]);
+    ea[j].guide = r.epf.guide;
     ea[j].xyb = r.xyb;
     ea[j].sigma = r.sigma;
     ea[j].epf_out = eo[eimg[j]];

@@ -280,6 +280,17 @@ __device__ __forceinline__ float guide_scaled(const SigmaParams& sp, int c, floa
   return __fmul_rn(__fsub_rn(v, sp.gmin[c]), sp.gscale[c]);
 }
 
+// J.2.2 guide byte of a scaled value, in the low 8 bits (others undefined):
+// clamped to [0, 255] and truncated by an addition of 2^23 that rounds toward
+// zero (the conversion unit has an eighth of the adders' rate).
+__device__ __forceinline__ uint32_t guide_byte(float s) {
+  return __float_as_uint(__fadd_rz(fminf(fmaxf(s, 0.f), 255.f), 8388608.f));
+}
+// The low bytes of four words.
+__device__ __forceinline__ uint32_t pack4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
+}
+
 // ---------------------------------------------------------------------------
 // k_validate
 // ---------------------------------------------------------------------------
@@ -761,23 +772,34 @@ __device__ void cell_sigma(float (*S)[kPR][kRS], CellState& cs, const SigmaParam
     const int lx0 = 8 * (b & 3), ly = 8 * (b >> 2) + r;
     const int gy = gby0 * 8 + ly;
     float rmax = -1.f;
-    bool any = false;
     float mn[3], mx[3];
+    // columns of the row inside the image (its samples take part in the range)
+    const int lim = gy < ys ? xs - (gbx0 * 8 + lx0) : 0;
+    bool any = lim > 0;
+    const bool store = epf.guide && gy < 8 * bh && gbx0 * 8 + lx0 < 8 * bw;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) { mn[c] = 3.0e38f; mx[c] = -3.0e38f; }
-    if (gy < ys) {
+    for (int c = 0; c < 3; ++c) {
+      const float4 v0 = *reinterpret_cast<const float4*>(&S[c][ly][lx0]);
+      const float4 v1 = *reinterpret_cast<const float4*>(&S[c][ly][lx0 + 4]);
+      float g[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int gx = gbx0 * 8 + lx0 + j;
-        if (gx < xs) {
-          any = true;
+      for (int j = 0; j < 8; ++j) g[j] = guide_scaled(sp, c, g[j]);
+      if (store) {
+        uint2 w;
+        w.x = pack4(guide_byte(g[0]), guide_byte(g[1]), guide_byte(g[2]), guide_byte(g[3]));
+        w.y = pack4(guide_byte(g[4]), guide_byte(g[5]), guide_byte(g[6]), guide_byte(g[7]));
+        *reinterpret_cast<uint2*>(epf.guide + c * epf.pps + static_cast<size_t>(gy) * epf.prs +
+                                  gbx0 * 8 + lx0) = w;
+      }
+      mn[c] = 3.0e38f;
+      mx[c] = -3.0e38f;
+      if (lim >= 8) {
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const float s = guide_scaled(sp, c, S[c][ly][lx0 + j]);
-            mn[c] = fminf(mn[c], s);
-            mx[c] = fmaxf(mx[c], s);
-          }
-        }
+        for (int j = 0; j < 8; ++j) { mn[c] = fminf(mn[c], g[j]); mx[c] = fmaxf(mx[c], g[j]); }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (j < lim) { mn[c] = fminf(mn[c], g[j]); mx[c] = fmaxf(mx[c], g[j]); }
       }
     }
 #pragma unroll
@@ -2486,36 +2508,44 @@ __global__ void __launch_bounds__(128, 4) k_epf(const __grid_constant__ FilterAr
 // output (k_epf_work_batch: the same for many images).
 //   k_epf_work  persistent one-warp CTAs taking 2 listed blocks at a time
 //               (a group; the warps claim groups from a per-request counter):
-//               per block a window of mirrored samples and packed guide
-//               bytes (6.5, J.2.2), the bytes then regrouped as planar words
-//               (4 neighbouring columns of one channel, one word per start
-//               column), so that one byte-SAD instruction takes 4 columns of
-//               a patch row.  A lane holds half a column of a block (4
-//               pixels): per horizontal offset it loads the 12 x 3 neighbour
-//               words once, forms the 6 patch-row sums of each of the 7
-//               vertical offsets (3 chained SADs each), adds 3 rows per
-//               pixel, and keeps the 28 patch SADs in registers for the warp
-//               votes (any of the 7 offsets live, then which) and for the
-//               live ones the weights and the J.2.5 sums.
+//               per block the J.2.2 guide bytes of its window, read from the
+//               planar bytes that the sigma pass stored (kPlane; mirrored
+//               windows at the image bounds byte by byte; without the plane
+//               from the samples), laid out as planar words (4 neighbouring
+//               columns of one channel, one word per start column), so that
+//               one byte-SAD instruction takes 4 columns of a patch row.  A
+//               lane holds half a column of a block (4 pixels): per horizontal
+//               offset it loads the 12 x 3 neighbour words once, forms the 6
+//               patch-row sums of each of the 7 vertical offsets (3 chained
+//               SADs each), adds 3 rows per pixel, and keeps the 28 patch SADs
+//               in registers for the warp votes (any of the 7 offsets live,
+//               then which) and for the live ones the weights and the J.2.5
+//               sums.  The sample windows those need come by asynchronous
+//               copies, issued before the guide words when the warp's last
+//               group needed them and else on the first live offset beyond
+//               the centre (noise-like content has only the centre live).
 //               Weights, cut-off and summation order are those of k_epf, so
 //               the two kernels give the same bits (an offset skipped by
 //               the vote would add exactly zero).  Warps synchronise only
 //               within themselves: a CTA never waits on another warp.
 //
 // Bound by the integer pipe (half rate: 126 SADs, 28 three-way adds and 17
-// minima per lane and horizontal offset) and, at 16 warps per SM, by the
-// latency of the window loads: ALU pipe 64% busy at 2048^2.  Against the
-// earlier form (one SAD per pixel, packed horizontal 4-sums through shared
-// memory, 16-bit loads back for the vertical sums: 13 instructions per pixel
-// and offset instead of 7.5) the whole step at 4096^2 takes 0.645 ms instead
-// of 0.717 (this kernel 0.307 -> 0.235), at 3001x2003 with most offsets live
-// 0.425 instead of 0.460.  A lane per whole column (8 pixels, 4 blocks per
-// warp) has 12% fewer instructions but only 8 warps per SM and takes longer
-// (0.692 and 0.555 ms for the same steps).
+// minima per lane and horizontal offset; 63% busy at 2048^2) and, at 16 warps
+// per SM, by the latency of each group's loads.  Measured steps (whole
+// request, 4096^2 with few live offsets / 3001x2003 photograph with most
+// live): one SAD per pixel and packed horizontal 4-sums through shared memory
+// (13 instructions per pixel and offset) 0.717 / 0.460 ms; planar words formed
+// from sample windows of every group 0.645 / 0.425 (this kernel 0.307 -> 0.235
+// at 4096^2); guide bytes stored once by the sigma pass (4.5 window samples per
+// pixel converted before, 3133 -> 2160 warp instructions per group) and sample
+// windows only on demand 0.602 / 0.417.  A lane per whole column (8 pixels, 4
+// blocks per warp) has 12% fewer instructions but only 8 warps per SM: 0.692
+// and 0.555 ms against 0.645 and 0.425.  Loading every window on demand cost
+// the photograph its latency (0.437 ms).
 // ---------------------------------------------------------------------------
 constexpr int kLG = 2;                            // blocks per warp and round (the lane
                                                   // layout of the sums assumes 2)
-constexpr int kLGH = 16, kLGW = 18, kLGS = 19;    // guide window, origin (-4, -4) of the block
+constexpr int kLGH = 16, kLGW = 18;               // guide window, origin (-4, -4) of the block
 constexpr int kLWC = 15, kLWS = 20;               // planar guide words: start columns, words per
                                                   // column (16 rows, 16-byte multiples)
 constexpr int kLWB = 912;                         // words per block (>= 3 kLWC kLWS, = 16 mod 32)
@@ -2536,14 +2566,15 @@ __device__ __forceinline__ uint32_t sad4(uint32_t a, uint32_t b, uint32_t acc) {
 
 // The groups of one image's list (total listed blocks) a warp takes: g0,
 // g0 + gs, ... or, with next (a zeroed counter), the ones it claims there one
-// at a time, the next claim issued before the current group's work.
-template <bool kClamp>
+// at a time, the next claim issued before the current group's work.  needed:
+// the warp's last group needed its sample windows (false at first).
+template <bool kClamp, bool kPlane>
 __device__ __forceinline__ void epf_work_groups(const FilterArgs& a, const int* __restrict__ list,
-                                                int total, int g0, int gs,
+                                                int total, int g0, int gs, bool& needed,
                                                 unsigned* next = nullptr) {
   __shared__ __align__(16) uint32_t W[kLG][kLWB];
   __shared__ float F[kLG][kLFB];
-  static_assert(kLGH * kLGS <= kLWB && 3 * kLWC * kLWS <= kLWB, "window sizes");
+  static_assert(kLGH * 16 <= kLWB && 3 * kLWC * kLWS <= kLWB, "window sizes");
   const int lane = threadIdx.x;
   const int C = 0x3F800000;
   const int T16 = static_cast<int>((a.wmin_bits + 0xFFFFu) & 0xFFFF0000u);
@@ -2559,71 +2590,88 @@ __device__ __forceinline__ void epf_work_groups(const FilterArgs& a, const int* 
     unsigned claim = 0;
     if (next && lane == 0) claim = atomicAdd(next, 1u);   // used after this group
     const int nb = min(kLG, total - kLG * grp);
-    // ---- windows of mirrored samples and packed guide bytes (6.5, J.2.2) --
+    // the group's blocks (the second one of an odd last group repeats the first)
+    const int b0 = __ldg(list + kLG * grp), b1 = __ldg(list + kLG * grp + nb - 1);
+    const int by0 = b0 / a.bw, bx0 = b0 - by0 * a.bw, by1 = b1 / a.bw, bx1 = b1 - by1 * a.bw;
+    // ---- mirrored (6.5) sample windows of the group's blocks, by asynchronous
+    // copies: lane = (every other row, column).  Needed only where an offset
+    // other than the centre is live: issued here when the warp's last group
+    // needed them, else when that is known ------------------------------------
+    auto load_windows = [&]() {
+#pragma unroll 1
+      for (int k = 0; k < kLG; ++k) {
+        const int wx0 = 8 * (k ? bx1 : bx0) - 3, wy0 = 8 * (k ? by1 : by0) - 3;
+        const int fc = lane & 15, f0 = lane >> 4;
+        if (fc < kLFW) {
+          const float* x = a.xyb + mirror_coord(wx0 + fc, a.xs);
 #pragma unroll
-    for (int k = 0; k < kLG; ++k) {
-      if (k >= nb) break;
-      const int b = __ldg(list + kLG * grp + k);
-      const int by = b / a.bw;
-      const int wx0 = 8 * (b - by * a.bw) - 4, wy0 = 8 * by - 4;
-      const bool inner = wx0 >= 0 && wy0 >= 0 && wx0 + kLGW <= a.xs && wy0 + kLGH <= a.ys;
-      constexpr int kPer = (kLGH * kLGW + 31) / 32;   // 9
-      float wv[kPer][3];
+          for (int i = 0; i < kLFH / 2; ++i) {
+            const int fr = 2 * i + f0;
+            const float* xr = x + static_cast<size_t>(mirror_coord(wy0 + fr, a.ys)) * a.rstride;
+            const uint32_t d = smem_addr(&F[k][fr * kLFS + lf_col(fr, fc)]);
 #pragma unroll
-      for (int q = 0; q < kPer; ++q) {
-        const int p = lane + 32 * q;
-        const int ly = p / kLGW, lx = p - ly * kLGW;
-        const int gy = inner ? wy0 + ly : mirror_coord(wy0 + ly, a.ys);
-        const int gx = inner ? wx0 + lx : mirror_coord(wx0 + lx, a.xs);
-        const size_t off = static_cast<size_t>(gy) * a.rstride + gx;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) wv[q][c] = __ldg(a.xyb + c * a.pstride + off);
-      }
-#pragma unroll
-      for (int q = 0; q < kPer; ++q) {
-        const int p = lane + 32 * q;
-        const int ly = p / kLGW, lx = p - ly * kLGW;
-        uint32_t g = 0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const float sc = fminf(fmaxf(guide_scaled(a.sp, c, wv[q][c]), 0.f), 255.f);
-          g |= static_cast<uint32_t>(sc) << (8 * c);
-        }
-        W[k][ly * kLGS + lx] = g;
-        if (ly >= 1 && ly <= kLFH && lx >= 1 && lx <= kLFW) {
-#pragma unroll
-          for (int c = 0; c < 3; ++c)
-            F[k][c * kLFC + (ly - 1) * kLFS + lf_col(ly - 1, lx - 1)] = wv[q][c];
+            for (int c = 0; c < 3; ++c)
+              asm volatile("cp.async.ca.shared.global [%0], [%1], 4;"
+                           :: "r"(d + 4 * c * kLFC), "l"(xr + c * a.pstride) : "memory");
+          }
         }
       }
-    }
-    __syncwarp();
+    };
+    if (needed) load_windows();
     // ---- planar guide words: lane = (block, window row); the word of channel
     // c at start column s holds that channel's bytes of columns s .. s + 3 ----
     {
       const int row = lane & 15;
       uint32_t* Wk = &W[lane >> 4][0];
-      uint32_t g[kLGW];
+      const int wx0 = 8 * (lane < 16 ? bx0 : bx1) - 4, wy0 = 8 * (lane < 16 ? by0 : by1) - 4;
+      const bool inner = wx0 >= 0 && wy0 >= 0 && wx0 + kLGW <= a.xs && wy0 + kLGH <= a.ys;
+      uint32_t A[3][5];      // the row's bytes, columns 0 .. 19 (18 used)
+      if (kPlane && __all_sync(0xFFFFFFFFu, inner)) {
+        const uint8_t* gp = a.guide + static_cast<size_t>(wy0 + row) * a.ors + wx0;
 #pragma unroll
-      for (int i = 0; i < kLGW; ++i) g[i] = Wk[row * kLGS + i];
-      __syncwarp();
+        for (int c = 0; c < 3; ++c)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        uint32_t w = __byte_perm(__byte_perm(g[0], g[1], c | (4 + c) << 4),
-                                 __byte_perm(g[2], g[3], c | (4 + c) << 4), 0x5410);
-        Wk[c * kLWC * kLWS + row] = w;
+          for (int i = 0; i < 5; ++i)
+            A[c][i] = __ldg(reinterpret_cast<const uint32_t*>(gp + c * a.ops) + i);
+      } else {
+        // mirrored (6.5) windows, sample by sample through shared memory
+        uint8_t* B = reinterpret_cast<uint8_t*>(&W[0][0]);
+#pragma unroll 6
+        for (int q = 0; q < kLG * kLGH * kLGW / 32; ++q) {
+          const int p = lane + 32 * q;
+          const int k = p / (kLGH * kLGW), r = p - k * (kLGH * kLGW);
+          const int ly = r / kLGW, lx = r - ly * kLGW;
+          const int gy = mirror_coord(8 * (k ? by1 : by0) - 4 + ly, a.ys);
+          const int gx = mirror_coord(8 * (k ? bx1 : bx0) - 4 + lx, a.xs);
 #pragma unroll
-        for (int s = 1; s < kLWC; ++s) {
-          w = __byte_perm(w, g[s + 3], 0x0321 | (4 + c) << 12);
-          Wk[(c * kLWC + s) * kLWS + row] = w;
+          for (int c = 0; c < 3; ++c) {
+            uint32_t g;
+            if (kPlane)
+              g = __ldg(a.guide + c * a.ops + static_cast<size_t>(gy) * a.ors + gx);
+            else
+              g = guide_byte(guide_scaled(
+                  a.sp, c, __ldg(a.xyb + c * a.pstride + static_cast<size_t>(gy) * a.rstride + gx)));
+            B[k * 4 * kLWB + ly * 64 + c * 20 + lx] = static_cast<uint8_t>(g);
+          }
         }
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+          for (int i = 0; i < 5; ++i) A[c][i] = Wk[row * 16 + c * 5 + i];
+        __syncwarp();
       }
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int s = 0; s < kLWC; ++s)
+          Wk[(c * kLWC + s) * kLWS + row] =
+              (s & 3) ? __funnelshift_r(A[c][s >> 2], A[c][(s >> 2) + 1], 8 * (s & 3)) : A[c][s >> 2];
     }
 
     // ---- this lane's half column -----------------------------------------
     const bool strip = sk < nb;
-    const int sb0 = strip ? __ldg(list + kLG * grp + sk) : 0;
-    const int sby = sb0 / a.bw, sbx = sb0 - sby * a.bw;
+    const int sb0 = sk ? b1 : b0, sby = sk ? by1 : by0, sbx = sk ? bx1 : bx0;
     int Mneg = 0, vmax = -1;
     if (strip) {
       const int sg = min(max(static_cast<int>(a.sigma[sb0]), 16), 672);
@@ -2636,6 +2684,8 @@ __device__ __forceinline__ void epf_work_groups(const FilterArgs& a, const int* 
     float2 ax[2], ay[2], ab[2], ws[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) ax[q] = ay[q] = ab[q] = ws[q] = make_float2(0.f, 0.f);
+    // whether the sample windows' copies to F were issued and have landed
+    bool issued = needed, landed = false;
     __syncwarp();
     // the lane's own words: columns cx - 1 .. cx + 2 of block rows r0 - 1 .. r0 + 4
     const uint32_t* Wl = &W[sk][cx * kLWS + r0];
@@ -2686,6 +2736,31 @@ __device__ __forceinline__ void epf_work_groups(const FilterArgs& a, const int* 
 #pragma unroll
       for (int oi = 0; oi < 7; ++oi) live |= static_cast<unsigned>(smin[oi] <= vmax) << oi;
       live = __reduce_or_sync(0xFFFFFFFFu, live);
+      if (!landed && g == 3 && live == 1u << 3) {
+        // the centre alone, whose weight is 1: the lane's own samples
+        const int gx = min(8 * sbx + cx, a.xs - 1);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          float v[3][2];
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            const float* x = a.xyb + static_cast<size_t>(min(8 * sby + r0 + 2 * q + r, a.ys - 1)) * a.rstride + gx;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) v[c][r] = __ldg(x + c * a.pstride);
+          }
+          ax[q] = __fadd2_rn(make_float2(v[0][0], v[0][1]), ax[q]);
+          ay[q] = __fadd2_rn(make_float2(v[1][0], v[1][1]), ay[q]);
+          ab[q] = __fadd2_rn(make_float2(v[2][0], v[2][1]), ab[q]);
+          ws[q] = __fadd2_rn(ws[q], make_float2(1.f, 1.f));
+        }
+        continue;
+      }
+      if (!landed) {
+        if (!issued) load_windows();
+        issued = landed = true;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+      }
       {
         const float* Fk = &F[sk][0];
         const int col = cx + ox + 3;
@@ -2743,17 +2818,21 @@ __device__ __forceinline__ void epf_work_groups(const FilterArgs& a, const int* 
         }
       }
     }
+    if (issued && !landed) asm volatile("cp.async.wait_all;" ::: "memory");
+    needed = landed;
     __syncwarp();   // the next group's windows overwrite W and F
     grp = next ? static_cast<int>(__shfl_sync(0xFFFFFFFFu, claim, 0)) : grp + gs;
   }
 }
 
-template <bool kClamp>
+template <bool kClamp, bool kPlane>
 __global__ void __launch_bounds__(32, 16) k_epf_work(const __grid_constant__ FilterArgs a,
                                                      const int* __restrict__ list,
                                                      const unsigned* __restrict__ count,
                                                      unsigned* next) {
-  epf_work_groups<kClamp>(a, list, static_cast<int>(*count), blockIdx.x, gridDim.x, next);
+  bool needed = false;
+  epf_work_groups<kClamp, kPlane>(a, list, static_cast<int>(*count), blockIdx.x, gridDim.x, needed,
+                                  next);
 }
 
 // Multi-image form: the groups of 2 listed blocks of all images, image after
@@ -2767,7 +2846,7 @@ __global__ void __launch_bounds__(32, 16) k_epf_work(const __grid_constant__ Fil
 // of listed blocks (args[j].epf_count points there).  The image's parameter
 // block is read where it is (warp-uniform loads through L1), so that the
 // shared memory of a warp is that of k_epf_work and as many warps fit.
-template <bool kClamp>
+template <bool kClamp, bool kPlane>
 __global__ void __launch_bounds__(32, 16) k_epf_work_batch(const FilterArgs* __restrict__ args,
                                                            const unsigned* __restrict__ counts,
                                                            int nimg, unsigned* next) {
@@ -2788,6 +2867,7 @@ __global__ void __launch_bounds__(32, 16) k_epf_work_batch(const FilterArgs* __r
   };
   load_chunk();
   unsigned v = 0;
+  bool needed = false;
   if (lane == 0) v = atomicAdd(next, 1u);
   long long g = __shfl_sync(full, v, 0);
   for (;;) {
@@ -2806,7 +2886,8 @@ __global__ void __launch_bounds__(32, 16) k_epf_work_batch(const FilterArgs* __r
     if (lane == 0) claim = atomicAdd(next, 1u);   // used after this group
     // exactly the group g - first of image c0 + j
     const FilterArgs& a = args[c0 + j];
-    epf_work_groups<kClamp>(a, a.epf_list, total, static_cast<int>(g) - first, total);
+    epf_work_groups<kClamp, kPlane>(a, a.epf_list, total, static_cast<int>(g) - first, total,
+                                    needed);
     g = __shfl_sync(full, claim, 0);
   }
 }
@@ -2866,9 +2947,10 @@ void launch_filter_batch_tma(const FilterArgs* args, const int* prefix, const vo
 }
 
 void launch_epf_work_batch(const FilterArgs* args, const unsigned* counts, int nimg, bool clamp,
-                           int grid, unsigned* next, cudaStream_t s) {
-  if (clamp) k_epf_work_batch<true><<<grid, 32, 0, s>>>(args, counts, nimg, next);
-  else k_epf_work_batch<false><<<grid, 32, 0, s>>>(args, counts, nimg, next);
+                           bool plane, int grid, unsigned* next, cudaStream_t s) {
+  auto* k = clamp ? (plane ? k_epf_work_batch<true, true> : k_epf_work_batch<true, false>)
+                  : (plane ? k_epf_work_batch<false, true> : k_epf_work_batch<false, false>);
+  k<<<grid, 32, 0, s>>>(args, counts, nimg, next);
 }
 
 // The kernels use static shared memory; ask for the largest carveout so the
@@ -2883,11 +2965,15 @@ static void prefer_shared_carveout() {
   cudaFuncSetAttribute(k_recon_batch, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
   cudaFuncSetAttribute(k_epf<false>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
   cudaFuncSetAttribute(k_epf<true>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
-  cudaFuncSetAttribute(k_epf_work_batch<false>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
-  cudaFuncSetAttribute(k_epf_work_batch<true>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+  cudaFuncSetAttribute(k_epf_work_batch<false, false>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+  cudaFuncSetAttribute(k_epf_work_batch<false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+  cudaFuncSetAttribute(k_epf_work_batch<true, false>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+  cudaFuncSetAttribute(k_epf_work_batch<true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
   cudaFuncSetAttribute(k_filter, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
-  cudaFuncSetAttribute(k_epf_work<false>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
-  cudaFuncSetAttribute(k_epf_work<true>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+  cudaFuncSetAttribute(k_epf_work<false, false>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+  cudaFuncSetAttribute(k_epf_work<false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+  cudaFuncSetAttribute(k_epf_work<true, false>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+  cudaFuncSetAttribute(k_epf_work<true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
   cudaGetLastError();
 }
 
@@ -2896,7 +2982,7 @@ int batch_blocks_per_sm(int kind) {
   cudaError_t e = cudaSuccess;
   if (kind == 0) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_recon_batch, 128, 0);
   else if (kind == 1)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_epf_work_batch<false>, 32, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_epf_work_batch<false, true>, 32, 0);
   else if (kind == 2)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_filter_batch, 256, 0);
   else
@@ -2919,11 +3005,13 @@ void launch_epf_work(const FilterArgs& a, const int* list, const unsigned* count
   if (grid == 0) {
     int sms = 0, per = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_epf_work<false>, 32, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_epf_work<false, true>, 32, 0);
     grid = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
   }
-  if (filter_needs_clamp(a)) k_epf_work<true><<<grid, 32, 0, s>>>(a, list, count, next);
-  else k_epf_work<false><<<grid, 32, 0, s>>>(a, list, count, next);
+  const bool clamp = filter_needs_clamp(a), plane = a.guide != nullptr;
+  auto* k = clamp ? (plane ? k_epf_work<true, true> : k_epf_work<true, false>)
+                  : (plane ? k_epf_work<false, true> : k_epf_work<false, false>);
+  k<<<grid, 32, 0, s>>>(a, list, count, next);
 }
 
 void launch_filter(const FilterArgs& a, cudaStream_t s) {

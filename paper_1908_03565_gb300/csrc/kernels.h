@@ -39,6 +39,8 @@ struct EpfSink {
   unsigned* count;
   float* pass;
   size_t prs, pps;
+  uint8_t* guide;             // J.2.2 guide bytes, planar [3][hp][prs] (8-byte aligned rows of
+                              // the padded width, planes pps apart), or nullptr: not stored
 };
 
 struct ReconArgs {
@@ -91,6 +93,8 @@ struct FilterArgs {
   OutParams out;
   float* epf_out;             // J.2 result (planar XYB) of k_epf_work,
   size_t ors, ops;            // row / plane stride in elements
+  const uint8_t* guide;       // J.2: the guide bytes the sigma pass stored (EpfSink; strides
+                              // ors / ops), or nullptr: formed from xyb
   const int* epf_list;        // multi-image J.2: the image's listed blocks and their
   const unsigned* epf_count;  // number (EpfSink of its sigma pass)
   unsigned* err;              // bounded device waits set bit 8 here on expiry (or nullptr)
@@ -158,8 +162,9 @@ void launch_filter_batch_tma(const FilterArgs* args, const int* prefix, const vo
 // pass copied the unchanged blocks), persistent grid of one-warp CTAs;
 // counts[i] is image i's listed-block count (args[i].epf_count == counts + i).
 // next: a zeroed counter the warps claim the groups of all images from.
+// plane: every args[i].guide is set (else none is).
 void launch_epf_work_batch(const FilterArgs* args, const unsigned* counts, int nimg, bool clamp,
-                           int grid, unsigned* next, cudaStream_t s);
+                           bool plane, int grid, unsigned* next, cudaStream_t s);
 // Work items (32x32 tiles) of k_filter for a, and whether the EPF needs its
 // exact-clamp variant for a's parameters.
 int filter_tiles(const FilterArgs& a);
