@@ -998,12 +998,16 @@ extern "C" jxlr_status jxl_recon_submit_jpeg(jxl_recon_ctx* ctx, const jxl_jpeg_
   }
   mark(slot, 1);
   mark(slot, 2);
-  JpegColorArgs ca;
+  JpegOutArgs ca;
   std::memset(&ca, 0, sizeof(ca));
+  JpegIdctArgs planes[3];   // components that go through a sample plane
+  int nplanes = 0;
+  JpegGabArgs gabs[3];
+  int ngabs = 0;
   for (int c = 0; c < nc; ++c) {
     const jxl_jpeg_component& k = st->comp[c];
     const int bw = static_cast<int>(k.width_in_blocks), bh = static_cast<int>(k.height_in_blocks);
-    JpegIdctArgs ia;
+    JpegIdctArgs& ia = ca.i[c];
     ia.coef = coef[c];
     ia.bw = bw;
     ia.bh = bh;
@@ -1039,11 +1043,12 @@ extern "C" jxlr_status jxl_recon_submit_jpeg(jxl_recon_ctx* ctx, const jxl_jpeg_
       ia.m0 = static_cast<float>(k.quant[0] / 8.0);
       ia.m1 = static_cast<float>(k.quant[0] / 8.0 / std::cos(3.14159265358979323846 / 16.0));
     }
-    launch_jpeg_idct(ia, s);
-    ctx->launches++;
     const float* plane = ia.plane;
+    const bool up = static_cast<int>(k.h_samp) != hmax || static_cast<int>(k.v_samp) != vmax;
+    ca.direct[c] = !up && !k.gab;
+    if (!ca.direct[c]) planes[nplanes++] = ia;
     if (k.gab) {
-      JpegGabArgs ga;
+      JpegGabArgs& ga = gabs[ngabs++];
       ga.src = ia.plane;
       ga.dst = cv.take<float>(static_cast<size_t>(bw) * bh * 64);
       ga.bw = bw;
@@ -1054,8 +1059,6 @@ extern "C" jxlr_status jxl_recon_submit_jpeg(jxl_recon_ctx* ctx, const jxl_jpeg_
       ga.w2n = static_cast<float>(k.gab_w2 / norm);
       ga.threshold = k.gab_threshold;
       ga.limit = k.gab_limit;
-      launch_jpeg_gab(ga, s);
-      ctx->launches++;
       plane = ga.dst;
     }
     ca.p[c].data = plane;
@@ -1063,6 +1066,14 @@ extern "C" jxlr_status jxl_recon_submit_jpeg(jxl_recon_ctx* ctx, const jxl_jpeg_
     ca.p[c].h = 8 * bh;
     ca.p[c].up_x = static_cast<int>(k.h_samp) != hmax;
     ca.p[c].up_y = static_cast<int>(k.v_samp) != vmax;
+  }
+  if (nplanes) {
+    launch_jpeg_idct(planes, nplanes, s);
+    ctx->launches++;
+  }
+  for (int g = 0; g < ngabs; ++g) {
+    launch_jpeg_gab(gabs[g], s);
+    ctx->launches++;
   }
   mark(slot, 3);
   ca.ncomp = nc;
@@ -1077,7 +1088,7 @@ extern "C" jxlr_status jxl_recon_submit_jpeg(jxl_recon_ctx* ctx, const jxl_jpeg_
   }
   ca.stride = out->row_stride_bytes;
   ca.dtype = out->dtype;
-  launch_jpeg_color(ca, s);
+  launch_jpeg_out(ca, s);
   ctx->launches++;
   mark(slot, 4);
   if (!out->on_device)

@@ -3,20 +3,38 @@
 //
 //  k_jpeg_cond_rows / k_jpeg_cond_cols  M.6.1.1 plateau scans, one thread
 //               per block row / column.
-//  k_jpeg_idct  128 threads = 16 blocks x 8 rows.  A thread loads one
-//               coefficient row (8 x int16, one 128-bit load), dequantises
-//               it with the prescaled table and transforms it; the block's
-//               transpose goes through shared memory within the warp (a
-//               block's 8 rows are 8 lanes of one warp), then the column
-//               transform and the row store.
+//  k_jpeg_idct  sample planes of the components that need one (subsampled, or
+//               with the M.6.3 side channel), all in one launch: 128 threads =
+//               16 blocks x 8 rows.  A thread loads one coefficient row (8 x
+//               int16, one 128-bit load), dequantises it with the prescaled
+//               table and transforms it; the block's transpose goes through
+//               shared memory within the warp (a block's 8 rows are 8 lanes of
+//               one warp), then the column transform and the row store.
 //  k_jpeg_gab   one 8x8 block per 64-thread CTA: J.4 on the plane (mirrored
 //               at its bounds), the M.6.3 count by __syncthreads_count, and
 //               the block's smoothed or original samples.
-//  k_jpeg_color one output pixel per thread: M.6.4 upsampling of the
-//               subsampled planes evaluated at the pixel (separable linear,
-//               weights 3/4 and 1/4), M.6.5, the output encoding.
+//  k_jpeg_out   one row of an 8x8 block of the image per thread: the samples of
+//               full-resolution components straight from their coefficients
+//               (the transform of k_jpeg_idct, without a plane in between), of
+//               the others from their planes with M.6.4 (separable linear,
+//               weights 3/4 and 1/4), then M.6.5 and the output encoding, 8
+//               pixels stored as 8- or 16-byte words where rows allow it.
+//
+//               k_jpeg_out_420 is the same for the usual 4:2:0 stream.
+//
+// Bound by the latency of the loads and by instruction issue (50% busy), not
+// by bandwidth: a 4:2:0 stream reads 2 bytes per sample, keeps its chroma
+// planes (8 bytes per 4 pixels) in L2 and writes 3 bytes per pixel.  Measured
+// at 4096^2, 4:2:0, u8 (whole request): 0.196 ms with a plane for every
+// component and one thread per output pixel, 0.108 with luma straight from
+// its coefficients and 8 pixels per thread (k_jpeg_out), 0.100 with the loads
+// of k_jpeg_out_420 a block row ahead.  The dequantisation table is read from
+// shared memory: indexed by the lane's row in constant memory, each of its
+// reads was replayed for 8 rows.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+
+#include <cstring>
 
 #include "jpeg1.h"
 
@@ -109,18 +127,26 @@ __global__ void __launch_bounds__(128) k_jpeg_cond_cols(const __grid_constant__ 
             a.out.v_slope, a.out.has_v);
 }
 
-__global__ void __launch_bounds__(128) k_jpeg_idct(const __grid_constant__ JpegIdctArgs a) {
-  __shared__ float sT[16][8][9];
-  const int tid = threadIdx.x;
-  const int lb = tid >> 3, r = tid & 7;
-  const int blk = blockIdx.x * 16 + lb;
-  const int nblk = a.bw * a.bh;
-  float x[8];
-  if (blk < nblk) {
-    const int4 raw = __ldg(reinterpret_cast<const int4*>(a.coef + static_cast<size_t>(blk) * 64 + 8 * r));
+// Row r (0..7) of the samples of block blk, in x, by the 8 threads of one warp
+// that hold the block's rows; on: the block exists (else zeros take part).  dq:
+// the component's prescaled table in shared memory; T: the block's scratch
+// (kBlockScratch floats, rows of 12: 16-byte row accesses and the column
+// accesses of a warp's 4 blocks without bank conflicts); raw: the coefficients
+// of row r.
+constexpr int kBlockScratch = 8 * 12 + 8;
+__device__ __forceinline__ int4 load_row(const JpegIdctArgs& a, int blk, int r, bool on) {
+  return on ? __ldg(reinterpret_cast<const int4*>(a.coef + static_cast<size_t>(blk) * 64 + 8 * r))
+            : make_int4(0, 0, 0, 0);
+}
+__device__ __forceinline__ void block_row(const JpegIdctArgs& a, const float* dq, float* T,
+                                          const int4& raw, int blk, int r, bool on, float (&x)[8]) {
+  if (on) {
     const int16_t* h = reinterpret_cast<const int16_t*>(&raw);
+    const float4 d0 = *reinterpret_cast<const float4*>(dq + 8 * r);
+    const float4 d1 = *reinterpret_cast<const float4*>(dq + 8 * r + 4);
+    const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
 #pragma unroll
-    for (int j = 0; j < 8; ++j) x[j] = static_cast<float>(h[j]) * a.dq[8 * r + j];
+    for (int j = 0; j < 8; ++j) x[j] = static_cast<float>(h[j]) * d[j];
     if (a.cond && r < 2) {   // M.6.1.1: coefficients 0 and 1 (row 0), 8 (row 1)
       const bool hh = a.c.has_h[blk] != 0, vh = a.c.has_v[blk] != 0;
       if (r == 0) {
@@ -141,22 +167,46 @@ __global__ void __launch_bounds__(128) k_jpeg_idct(const __grid_constant__ JpegI
   // row r holds the coefficients of vertical frequency r: transform along
   // the horizontal frequencies first
   idct8(x);
-#pragma unroll
-  for (int j = 0; j < 8; ++j) sT[lb][r][j] = x[j];
+  float4* row = reinterpret_cast<float4*>(T + 12 * r);
+  row[0] = make_float4(x[0], x[1], x[2], x[3]);
+  row[1] = make_float4(x[4], x[5], x[6], x[7]);
   __syncwarp();
   // column r: the vertical transform of horizontal position r
 #pragma unroll
-  for (int j = 0; j < 8; ++j) x[j] = sT[lb][j][r];
+  for (int j = 0; j < 8; ++j) x[j] = T[12 * j + r];
   idct8(x);
   __syncwarp();
 #pragma unroll
-  for (int j = 0; j < 8; ++j) sT[lb][j][r] = x[j];
+  for (int j = 0; j < 8; ++j) T[12 * j + r] = x[j];
   __syncwarp();
+  const float4 lo = row[0], hi = row[1];
+  x[0] = lo.x; x[1] = lo.y; x[2] = lo.z; x[3] = lo.w;
+  x[4] = hi.x; x[5] = hi.y; x[6] = hi.z; x[7] = hi.w;
+  __syncwarp();   // the caller may transform another component's block
+}
+
+struct JpegIdctSet {
+  JpegIdctArgs c[3];
+};
+
+__global__ void __launch_bounds__(128) k_jpeg_idct(const __grid_constant__ JpegIdctSet set) {
+  const JpegIdctArgs& a = set.c[blockIdx.y];
+  __shared__ __align__(16) float sT[16][kBlockScratch];
+  __shared__ __align__(16) float s_dq[64];
+  const int tid = threadIdx.x;
+  const int lb = tid >> 3, r = tid & 7;
+  const int blk = blockIdx.x * 16 + lb;
+  const int nblk = a.bw * a.bh;
+  if (blockIdx.x * 16 >= nblk) return;
+  if (tid < 64) s_dq[tid] = a.dq[tid];
+  __syncthreads();
+  float x[8];
+  block_row(a, s_dq, sT[lb], load_row(a, blk, r, blk < nblk), blk, r, blk < nblk, x);
   if (blk < nblk) {
     const int by = blk / a.bw, bx = blk - by * a.bw;
     float* dst = a.plane + static_cast<size_t>(8 * by + r) * (8 * a.bw) + 8 * bx;
-    reinterpret_cast<float4*>(dst)[0] = make_float4(sT[lb][r][0], sT[lb][r][1], sT[lb][r][2], sT[lb][r][3]);
-    reinterpret_cast<float4*>(dst)[1] = make_float4(sT[lb][r][4], sT[lb][r][5], sT[lb][r][6], sT[lb][r][7]);
+    reinterpret_cast<float4*>(dst)[0] = make_float4(x[0], x[1], x[2], x[3]);
+    reinterpret_cast<float4*>(dst)[1] = make_float4(x[4], x[5], x[6], x[7]);
   }
 }
 
@@ -215,36 +265,177 @@ __device__ __forceinline__ float sample_up(const JpegPlane& p, int x, int y) {
   return fmaf(0.75f, h0, 0.25f * h1);
 }
 
-__global__ void __launch_bounds__(256) k_jpeg_color(const __grid_constant__ JpegColorArgs a) {
-  const int x = blockIdx.x * 32 + (threadIdx.x & 31);
-  const int y = blockIdx.y * 8 + (threadIdx.x >> 5);
-  if (x >= a.xs || y >= a.ys) return;
-  float r, g, b;
-  const float yv = sample_up(a.p[0], x, y) + 128.f;
-  if (a.ncomp == 1) {
-    r = g = b = yv;
-  } else {
-    const float cb = sample_up(a.p[1], x, y), cr = sample_up(a.p[2], x, y);
-    r = fmaf(1.402f, cr, yv);
-    g = fmaf(-0.71414f, cr, fmaf(-0.34414f, cb, yv));
-    b = fmaf(1.772f, cb, yv);
+// The 8 samples of pixels x .. x + 7 (x a multiple of 8) of image row y from
+// p's plane; columns at xs and beyond are not used (n of them are inside).
+__device__ __forceinline__ void plane_row(const JpegPlane& p, int x, int y, int n, float (&v)[8]) {
+  if (!p.up_x && !p.up_y) {
+    const float4* s = reinterpret_cast<const float4*>(p.data + static_cast<size_t>(y) * p.w + x);
+    const float4 a = __ldg(s), b = __ldg(s + 1);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) v[j] = j < n ? sample_up(p, x + j, y) : 0.f;
+}
+
+// M.6.5, M.6.6 and the output encoding of pixels x .. x + n - 1 (n <= 8) of row y.
+__device__ __forceinline__ void color_row(const JpegOutArgs& a, int x, int y, int n,
+                                          const float (&v)[3][8]) {
+  float o[24];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const float yv = v[0][j] + 128.f;
+    if (a.ncomp == 1) {
+      o[3 * j] = o[3 * j + 1] = o[3 * j + 2] = yv;
+    } else {
+      const float cb = v[1][j], cr = v[2][j];
+      o[3 * j] = fmaf(1.402f, cr, yv);
+      o[3 * j + 1] = fmaf(-0.71414f, cr, fmaf(-0.34414f, cb, yv));
+      o[3 * j + 2] = fmaf(1.772f, cb, yv);
+    }
   }
   char* row = static_cast<char*>(a.out) + static_cast<size_t>(y) * a.stride;
-  if (a.dtype == 2) {   // u8: clamp, round half up
-    uint8_t* o = reinterpret_cast<uint8_t*>(row) + 3 * x;
-    o[0] = static_cast<uint8_t>(floorf(fminf(fmaxf(r, 0.f), 255.f) + 0.5f));
-    o[1] = static_cast<uint8_t>(floorf(fminf(fmaxf(g, 0.f), 255.f) + 0.5f));
-    o[2] = static_cast<uint8_t>(floorf(fminf(fmaxf(b, 0.f), 255.f) + 0.5f));
-  } else if (a.dtype == 1) {
-    __half* o = reinterpret_cast<__half*>(row) + 3 * x;
-    o[0] = __float2half_rn(r * (1.f / 255.f));
-    o[1] = __float2half_rn(g * (1.f / 255.f));
-    o[2] = __float2half_rn(b * (1.f / 255.f));
+  if (a.dtype == 2) {   // u8: clamp, round half up (truncated by adding 2^23 toward zero)
+    uint32_t w[24];
+#pragma unroll
+    for (int k = 0; k < 24; ++k)
+      w[k] = __float_as_uint(__fadd_rz(fminf(fmaxf(o[k], 0.f), 255.f) + 0.5f, 8388608.f));
+    uint8_t* p = reinterpret_cast<uint8_t*>(row) + 3 * x;
+    if (n == 8 && (reinterpret_cast<uintptr_t>(p) & 7) == 0) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        uint32_t d[2];
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+          const uint32_t* q = w + 8 * k + 4 * m;
+          d[m] = __byte_perm(__byte_perm(q[0], q[1], 0x0040), __byte_perm(q[2], q[3], 0x0040), 0x5410);
+        }
+        reinterpret_cast<uint2*>(p)[k] = make_uint2(d[0], d[1]);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 24; ++k)
+        if (k < 3 * n) p[k] = static_cast<uint8_t>(w[k]);
+    }
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < 24; ++k) o[k] *= 1.f / 255.f;
+  if (a.dtype == 1) {
+    __half* p = reinterpret_cast<__half*>(row) + 3 * x;
+    if (n == 8 && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        uint32_t d[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const __half2 h = __floats2half2_rn(o[8 * k + 2 * m], o[8 * k + 2 * m + 1]);
+          d[m] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+        reinterpret_cast<uint4*>(p)[k] = make_uint4(d[0], d[1], d[2], d[3]);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 24; ++k)
+        if (k < 3 * n) p[k] = __float2half_rn(o[k]);
+    }
   } else {
-    float* o = reinterpret_cast<float*>(row) + 3 * x;
-    o[0] = r * (1.f / 255.f);
-    o[1] = g * (1.f / 255.f);
-    o[2] = b * (1.f / 255.f);
+    float* p = reinterpret_cast<float*>(row) + 3 * x;
+    if (n == 8 && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+#pragma unroll
+      for (int k = 0; k < 24; k += 4)
+        *reinterpret_cast<float4*>(p + k) = make_float4(o[k], o[k + 1], o[k + 2], o[k + 3]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 24; ++k)
+        if (k < 3 * n) p[k] = o[k];
+    }
+  }
+}
+
+__global__ void __launch_bounds__(128) k_jpeg_out(const __grid_constant__ JpegOutArgs a) {
+  __shared__ __align__(16) float sT[16][kBlockScratch];
+  __shared__ __align__(16) float s_dq[3][64];
+  const int tid = threadIdx.x;
+  const int lb = tid >> 3, r = tid & 7;
+  for (int k = tid; k < 64 * a.ncomp; k += 128)
+    if (a.direct[k >> 6]) s_dq[k >> 6][k & 63] = a.i[k >> 6].dq[k & 63];
+  __syncthreads();
+  const int bx = blockIdx.x * 16 + lb, x = 8 * bx, y = 8 * blockIdx.y + r;
+  const bool in = x < a.xs;                    // the block has pixels (the same for its 8 rows)
+  const int n = in && y < a.ys ? min(8, a.xs - x) : 0;
+  float v[3][8];
+  // all loads before the first transform
+  int4 raw[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    if (c < a.ncomp && a.direct[c]) raw[c] = load_row(a.i[c], blockIdx.y * a.i[c].bw + bx, r, in);
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    if (c < a.ncomp && !a.direct[c] && n > 0) plane_row(a.p[c], x, y, n, v[c]);
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    if (c < a.ncomp && a.direct[c])
+      block_row(a.i[c], s_dq[c], sT[lb], raw[c], blockIdx.y * a.i[c].bw + bx, r, in, v[c]);
+  if (n == 0) return;
+  color_row(a, x, y, n, v);
+}
+
+// The usual form, 4:2:0 without the side channels of M.6.3: luma direct, both
+// chroma components upsampled along both axes.  A CTA takes kRows420 block
+// rows of 16 blocks, the next row's coefficients loaded before the current
+// one's transform and the chroma samples before the luma transform.
+constexpr int kRows420 = 4;
+__global__ void __launch_bounds__(128) k_jpeg_out_420(const __grid_constant__ JpegOutArgs a) {
+  __shared__ __align__(16) float sT[16][kBlockScratch];
+  __shared__ __align__(16) float s_dq[64];
+  const int tid = threadIdx.x;
+  const int lb = tid >> 3, r = tid & 7;
+  const int bx = blockIdx.x * 16 + lb, x = 8 * bx;
+  const bool in = x < a.xs;
+  int by = blockIdx.y * kRows420;
+  const int by1 = min(by + kRows420, (a.ys + 7) >> 3);
+  int4 next = load_row(a.i[0], by * a.i[0].bw + bx, r, in);
+  if (tid < 64) s_dq[tid] = a.i[0].dq[tid];
+  __syncthreads();
+  // columns i0 - 1 .. i0 + 4 of the chroma planes, the outer ones mirrored (M.6.4)
+  const int w = a.p[1].w, i0 = in ? x >> 1 : 0;
+  const int left = i0 > 0 ? i0 - 1 : 1, right = i0 + 4 < w ? i0 + 4 : w - 2;
+  for (; by < by1; ++by) {
+    const int4 raw = next;
+    const int y = 8 * by + r;
+    const int n = in && y < a.ys ? min(8, a.xs - x) : 0;
+    if (by + 1 < by1) next = load_row(a.i[0], (by + 1) * a.i[0].bw + bx, r, in);
+    int y0 = 0, y1 = 0;
+    if (n) up_taps(y, a.p[1].h, y0, y1);
+    float ch[2][2][6];
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const float* row = a.p[1 + c].data + static_cast<size_t>(k ? y1 : y0) * w;
+        const float4 m = __ldg(reinterpret_cast<const float4*>(row + i0));
+        ch[c][k][0] = __ldg(row + left);
+        ch[c][k][1] = m.x; ch[c][k][2] = m.y; ch[c][k][3] = m.z; ch[c][k][4] = m.w;
+        ch[c][k][5] = __ldg(row + right);
+      }
+    float v[3][8];
+    block_row(a.i[0], s_dq, sT[lb], raw, by * a.i[0].bw + bx, r, in, v[0]);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      float h[2][8];
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          h[k][2 * j] = fmaf(0.75f, ch[c][k][j + 1], 0.25f * ch[c][k][j]);
+          h[k][2 * j + 1] = fmaf(0.75f, ch[c][k][j + 1], 0.25f * ch[c][k][j + 2]);
+        }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[1 + c][j] = fmaf(0.75f, h[0][j], 0.25f * h[1][j]);
+    }
+    if (n) color_row(a, x, y, n, v);
   }
 }
 
@@ -256,9 +447,16 @@ bool upload_jpeg_constants(const float* odd8, const float* odd4, float odd2) {
          cudaMemcpyToSymbol(c_jodd2, &odd2, sizeof(float)) == cudaSuccess;
 }
 
-void launch_jpeg_idct(const JpegIdctArgs& a, cudaStream_t s) {
-  const int nblk = a.bw * a.bh;
-  k_jpeg_idct<<<(nblk + 15) / 16, 128, 0, s>>>(a);
+void launch_jpeg_idct(const JpegIdctArgs* a, int n, cudaStream_t s) {
+  JpegIdctSet set;
+  std::memset(&set, 0, sizeof(set));
+  int most = 1;
+  for (int c = 0; c < n; ++c) {
+    set.c[c] = a[c];
+    const int nblk = a[c].bw * a[c].bh;
+    most = nblk > most ? nblk : most;
+  }
+  k_jpeg_idct<<<dim3((most + 15) / 16, n), 128, 0, s>>>(set);
 }
 
 int launch_jpeg_cond(const JpegCondArgs& a, cudaStream_t s) {
@@ -271,8 +469,14 @@ void launch_jpeg_gab(const JpegGabArgs& a, cudaStream_t s) {
   k_jpeg_gab<<<dim3(a.bw, a.bh), 64, 0, s>>>(a);
 }
 
-void launch_jpeg_color(const JpegColorArgs& a, cudaStream_t s) {
-  k_jpeg_color<<<dim3((a.xs + 31) / 32, (a.ys + 7) / 8), 256, 0, s>>>(a);
+void launch_jpeg_out(const JpegOutArgs& a, cudaStream_t s) {
+  const auto both = [&](int c) { return !a.direct[c] && a.p[c].up_x && a.p[c].up_y; };
+  const int rows = (a.ys + 7) / 8;
+  if (a.ncomp == 3 && a.direct[0] && both(1) && both(2) && a.p[1].w == a.p[2].w &&
+      a.p[1].h == a.p[2].h)
+    k_jpeg_out_420<<<dim3((a.xs + 127) / 128, (rows + kRows420 - 1) / kRows420), 128, 0, s>>>(a);
+  else
+    k_jpeg_out<<<dim3((a.xs + 127) / 128, rows), 128, 0, s>>>(a);
 }
 
 }  // namespace jxlr

@@ -51,7 +51,12 @@ struct JpegPlane {
   int up_x, up_y;             // 2x upsampling along x / y (M.6.4)
 };
 
-struct JpegColorArgs {
+// M.6.4 - M.6.6 with M.6.1 / M.6.2 of the components that need no plane:
+// direct[c] set, component c's samples come straight from its coefficients
+// (i[c]; i[c].plane unused), else from p[c].
+struct JpegOutArgs {
+  int direct[3];
+  JpegIdctArgs i[3];
   JpegPlane p[3];
   int ncomp;                  // 1 (grey) or 3 (YCbCr)
   int xs, ys;
@@ -61,11 +66,12 @@ struct JpegColorArgs {
 };
 
 bool upload_jpeg_constants(const float* odd8, const float* odd4, float odd2);
-void launch_jpeg_idct(const JpegIdctArgs& a, cudaStream_t s);
+// Sample planes of n (1..3) components, one launch.
+void launch_jpeg_idct(const JpegIdctArgs* a, int n, cudaStream_t s);
 // M.6.1.1 plateau scans: one thread per block row, then one per block
 // column; returns the number of launches.
 int launch_jpeg_cond(const JpegCondArgs& a, cudaStream_t s);
 void launch_jpeg_gab(const JpegGabArgs& a, cudaStream_t s);
-void launch_jpeg_color(const JpegColorArgs& a, cudaStream_t s);
+void launch_jpeg_out(const JpegOutArgs& a, cudaStream_t s);
 
 }  // namespace jxlr
