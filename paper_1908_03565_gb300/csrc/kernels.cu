@@ -202,13 +202,28 @@ __device__ __forceinline__ void xyb_to_rgb01_x2(const ColorParams& cp, float2 X,
   b = __ffma2_rn(f2(cp.m[6]), mr, __ffma2_rn(f2(cp.m[7]), mg, __fmul2_rn(f2(cp.m[8]), mb)));
 }
 
+// The low bytes of four words.
+__device__ __forceinline__ uint32_t pack4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
+}
+
+// IEC 61966-2-1 byte of a linear sample, in the low 8 bits (others undefined).
+// x^(1/2.4) as exp2(log2(x) / 2.4) with the hardware approximations: a few
+// ulps, far inside the 8-bit step.  No argument of the kept branch is denormal
+// (x above 0.0031, exponents in [-3.5, 0]), so the forms without denormal
+// handling give the same bits; the rounding down is an addition of 2^23 that
+// rounds toward zero: the two approximations are all that a sample asks of the
+// special-function unit (an eighth of the adders' rate).  With floor and the
+// conversion there too, 8-bit requests took 2.196 instead of 2.148 ms at
+// 8192^2 and 0.132 instead of 0.125 at 1920x1088; all 2^32 inputs give the same
+// byte either way.
 __device__ __forceinline__ uint32_t srgb8(float v) {
-  float x = fminf(fmaxf(v, 0.f), 1.f);
-  // x^(1/2.4) as exp2(log2(x) / 2.4) with the hardware approximations: a
-  // few ulps, far inside the 8-bit step
-  float e = x <= 0.0031308f ? 12.92f * x
-                            : fmaf(1.055f, exp2f(__log2f(x) * (1.f / 2.4f)), -0.055f);
-  return static_cast<uint32_t>(floorf(fmaf(e, 255.f, 0.5f)));
+  const float x = fminf(fmaxf(v, 0.f), 1.f);
+  float l, p;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(x));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(l * (1.f / 2.4f)));
+  const float e = x <= 0.0031308f ? 12.92f * x : fmaf(1.055f, p, -0.055f);
+  return __float_as_uint(__fadd_rz(fmaf(e, 255.f, 0.5f), 8388608.f));
 }
 
 // Stores n (1..4) consecutive pixels of one row starting at column px.
@@ -245,8 +260,7 @@ __device__ __forceinline__ void store_px4(const OutParams& o, int px, int py, co
       uint32_t* q = reinterpret_cast<uint32_t*>(p);
 #pragma unroll
       for (int k = 0; k < 3; ++k)
-        q[k] = srgb8(v[4 * k]) | (srgb8(v[4 * k + 1]) << 8) | (srgb8(v[4 * k + 2]) << 16) |
-               (srgb8(v[4 * k + 3]) << 24);
+        q[k] = pack4(srgb8(v[4 * k]), srgb8(v[4 * k + 1]), srgb8(v[4 * k + 2]), srgb8(v[4 * k + 3]));
     } else {
       for (int i = 0; i < 3 * n; ++i) p[i] = static_cast<uint8_t>(srgb8(v[i]));
     }
@@ -286,11 +300,6 @@ __device__ __forceinline__ float guide_scaled(const SigmaParams& sp, int c, floa
 __device__ __forceinline__ uint32_t guide_byte(float s) {
   return __float_as_uint(__fadd_rz(fminf(fmaxf(s, 0.f), 255.f), 8388608.f));
 }
-// The low bytes of four words.
-__device__ __forceinline__ uint32_t pack4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
-}
-
 // ---------------------------------------------------------------------------
 // k_validate
 // ---------------------------------------------------------------------------
