@@ -239,7 +239,9 @@ __device__ __forceinline__ void store_px4(const OutParams& o, int px, int py, co
       q[1] = make_float4(v[4], v[5], v[6], v[7]);
       q[2] = make_float4(v[8], v[9], v[10], v[11]);
     } else {
-      for (int i = 0; i < 3 * n; ++i) p[i] = v[i];
+#pragma unroll
+      for (int i = 0; i < 12; ++i)
+        if (i < 3 * n) p[i] = v[i];
     }
   } else if (o.dtype == 1) {
     __half* p = reinterpret_cast<__half*>(row) + 3 * px;
@@ -252,7 +254,9 @@ __device__ __forceinline__ void store_px4(const OutParams& o, int px, int py, co
         q[k] = make_uint2(*reinterpret_cast<uint32_t*>(&h0), *reinterpret_cast<uint32_t*>(&h1));
       }
     } else {
-      for (int i = 0; i < 3 * n; ++i) p[i] = __float2half_rn(v[i]);
+#pragma unroll
+      for (int i = 0; i < 12; ++i)
+        if (i < 3 * n) p[i] = __float2half_rn(v[i]);
     }
   } else {
     uint8_t* p = reinterpret_cast<uint8_t*>(row) + 3 * px;
@@ -262,7 +266,9 @@ __device__ __forceinline__ void store_px4(const OutParams& o, int px, int py, co
       for (int k = 0; k < 3; ++k)
         q[k] = pack4(srgb8(v[4 * k]), srgb8(v[4 * k + 1]), srgb8(v[4 * k + 2]), srgb8(v[4 * k + 3]));
     } else {
-      for (int i = 0; i < 3 * n; ++i) p[i] = static_cast<uint8_t>(srgb8(v[i]));
+#pragma unroll
+      for (int i = 0; i < 12; ++i)
+        if (i < 3 * n) p[i] = static_cast<uint8_t>(srgb8(v[i]));
     }
   }
 }
@@ -2150,60 +2156,97 @@ __device__ __forceinline__ void epf_tile(const FilterArgs& a, int tbx, int tby) 
 }
 
 // ---------------------------------------------------------------------------
-// J.4 Gaborish (optional) + K.5 + L.2 + store: 32x32 tile, 256 threads.  The
-// tile and a one-sample ring (mirrored at the image bounds, 6.5) are loaded
-// with all of a thread's loads in flight; each thread then takes 4
-// neighbouring pixels of one row (6 x 3 samples per channel as one 16-byte
-// and one 8-byte shared load per row) and stores them as 16-byte words.
+// J.4 Gaborish (optional) + K.5 + L.2 + store of a 32x32 tile.  The tile and
+// its ring (one sample, mirrored at the image bounds, 6.5) lie in shared
+// memory, in rows of kQW floats whose first tile column is at 4; each thread
+// takes 4 neighbouring pixels of R rows (256 / R threads).
+//
+// Bound by instruction issue and latencies next to memory (the floor is 24
+// bytes a pixel with f32 output: 59 us at 4096^2).  With two rows a thread,
+// the centre and the left + right sum of each of the four rows it touches are
+// formed once; the outer columns of a 4-column group come from the
+// neighbouring lanes (a scalar load of every fourth column is replayed four
+// times for bank conflicts), and the pixels' values stay in registers (the
+// stores of a partial group indexed them, which kept them in local memory, 12
+// bytes written a pixel).  Whole requests, 92 instructions a pixel before: 4096^2
+// f32 0.600 -> 0.583 ms, 8192^2 u8 2.148 -> 2.095.  One row a thread: 0.593 and
+// 2.150; it is kept for the noise step, whose loads want the warps (2047x1535
+// with J.3 and noise 0.392 ms, two rows 0.414), and where the tile comes by
+// ordinary loads.
 // ---------------------------------------------------------------------------
-constexpr int kGT = 32, kGR = kGT + 2, kGS2 = 36;   // rows of 16-byte aligned 144 bytes
+constexpr int kGT = 32;
+constexpr int kQW = 40, kQH = 34;                          // tile with its ring (columns, rows)
 
-// J.4 (optional), K.5 and L.2 of the pixels gx .. gx + n - 1 (n <= 4) of row
-// gy from their neighbourhood w[c][r][i] (image row gy - 1 + r, column
-// gx - 1 + i), then the store.
-__device__ __forceinline__ void gab4_finish(const FilterArgs& a, int gx, int gy, int n,
-                                            const float (&w)[3][3][6]) {
-  float o[3][4];
+struct __align__(128) QTile {
+  float s[3][kQH][kQW];
+};
+
+// The tile at (x0, y0), its ring in place.
+template <int R>
+__device__ __forceinline__ void gab_pixels(const FilterArgs& a, const QTile& q, int x0, int y0) {
+  const int tid = threadIdx.x;
+  const int tx4 = tid & 7, ty = R * (tid >> 3);   // columns 4 tx4 .. 4 tx4 + 3, rows from ty
+  const unsigned full = 0xFFFFFFFFu;
+  float o[R][3][4];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    // pixels p and p + 1 as pairs
+    // rows ty - 1 .. ty + 2: the samples m and the left + right sums s, as pairs
+    float2 m[R + 2][2], s[R + 2][2];
 #pragma unroll
-    for (int p = 0; p < 4; p += 2) {
-      auto at = [&](int r, int i) { return make_float2(w[c][r][i], w[c][r][i + 1]); };
-      const float2 centre = at(1, p + 1);
-      float2 v = centre;
-      if (a.gab) {
-        const float2 edge = __fadd2_rn(__fadd2_rn(at(0, p + 1), at(2, p + 1)),
-                                       __fadd2_rn(at(1, p), at(1, p + 2)));
-        const float2 corner = __fadd2_rn(__fadd2_rn(at(0, p), at(0, p + 2)),
-                                         __fadd2_rn(at(2, p), at(2, p + 2)));
-        v = __ffma2_rn(f2(a.gw[c][0]), centre,
-                       __ffma2_rn(f2(a.gw[c][1]), edge, __fmul2_rn(f2(a.gw[c][2]), corner)));
-      }
-      o[c][p] = v.x;
-      o[c][p + 1] = v.y;
+    for (int k = 0; k < R + 2; ++k) {
+      const float* row = &q.s[c][ty + k][4 * tx4 + 4];
+      const float4 f = *reinterpret_cast<const float4*>(row);
+      float l = __shfl_up_sync(full, f.w, 1, 8), r = __shfl_down_sync(full, f.x, 1, 8);
+      if (tx4 == 0) l = row[-1];
+      if (tx4 == 7) r = row[4];
+      m[k][0] = make_float2(f.x, f.y);
+      m[k][1] = make_float2(f.z, f.w);
+      s[k][0] = make_float2(__fadd_rn(l, f.y), __fadd_rn(f.x, f.z));
+      s[k][1] = make_float2(__fadd_rn(f.y, f.w), __fadd_rn(f.z, r));
     }
-  }
-  if (a.noise) {
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
-      if (p < n) apply_noise(a, gx + p, gy, o[0][p], o[1][p], o[2][p]);
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        float2 v = m[i + 1][p];
+        if (a.gab) {
+          const float2 edge = __fadd2_rn(__fadd2_rn(m[i][p], m[i + 2][p]), s[i + 1][p]);
+          const float2 corner = __fadd2_rn(s[i][p], s[i + 2][p]);
+          v = __ffma2_rn(f2(a.gw[c][0]), v,
+                         __ffma2_rn(f2(a.gw[c][1]), edge, __fmul2_rn(f2(a.gw[c][2]), corner)));
+        }
+        o[i][c][2 * p] = v.x;
+        o[i][c][2 * p + 1] = v.y;
+      }
   }
-  emit4(a.cp, a.out, gx, gy, n, o[0], o[1], o[2]);
+  const int gx = x0 + 4 * tx4;
+  if (gx >= a.xs) return;
+  const int n = min(4, a.xs - gx);
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int gy = y0 + ty + i;
+    if (gy >= a.ys) break;
+    if (a.noise) {
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+        if (p < n) apply_noise(a, gx + p, gy, o[i][0][p], o[i][1][p], o[i][2][p]);
+    }
+    emit4(a.cp, a.out, gx, gy, n, o[i][0], o[i][1], o[i][2]);
+  }
 }
 
 __device__ __forceinline__ void gab_tile(const FilterArgs& a, int tbx, int tby) {
-  __shared__ __align__(16) float Wn[3][kGR][kGS2];
+  __shared__ QTile q;
   const int tid = threadIdx.x;
   const int x0 = tbx * kGT, y0 = tby * kGT;
   const bool inner = x0 >= 1 && y0 >= 1 && x0 + kGT + 1 <= a.xs && y0 + kGT + 1 <= a.ys;
-  constexpr int kN = kGR * kGR, kPer = (kN + 255) / 256;
+  constexpr int kW = kGT + 2, kN = kW * kQH, kPer = (kN + 256 - 1) / 256;
   float v[kPer][3];
 #pragma unroll
   for (int j = 0; j < kPer; ++j) {
     const int i = tid + 256 * j;
     if (i < kN) {
-      const int ly = i / kGR, lx = i - ly * kGR;
+      const int ly = i / kW, lx = i - ly * kW;
       const int gy = inner ? y0 - 1 + ly : mirror_coord(y0 - 1 + ly, a.ys);
       const int gx = inner ? x0 - 1 + lx : mirror_coord(x0 - 1 + lx, a.xs);
       const size_t off = static_cast<size_t>(gy) * a.rstride + gx;
@@ -2215,27 +2258,13 @@ __device__ __forceinline__ void gab_tile(const FilterArgs& a, int tbx, int tby) 
   for (int j = 0; j < kPer; ++j) {
     const int i = tid + 256 * j;
     if (i < kN) {
-      const int ly = i / kGR, lx = i - ly * kGR;
+      const int ly = i / kW, lx = i - ly * kW;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) Wn[c][ly][lx] = v[j][c];
+      for (int c = 0; c < 3; ++c) q.s[c][ly][lx + 3] = v[j][c];
     }
   }
   __syncthreads();
-  const int tx4 = tid & 7, ty = tid >> 3;   // pixels 4 tx4 .. 4 tx4 + 3 of row ty
-  const int gx = x0 + 4 * tx4, gy = y0 + ty;
-  if (gx >= a.xs || gy >= a.ys) return;
-  float w[3][3][6];   // window rows ty .. ty + 2 (image rows gy - 1 .. gy + 1), columns 4 tx4 ..
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      const float4 q = *reinterpret_cast<const float4*>(&Wn[c][ty + r][4 * tx4]);
-      const float2 e = *reinterpret_cast<const float2*>(&Wn[c][ty + r][4 * tx4 + 4]);
-      w[c][r][0] = q.x; w[c][r][1] = q.y; w[c][r][2] = q.z; w[c][r][3] = q.w;
-      w[c][r][4] = e.x; w[c][r][5] = e.y;
-    }
-  }
-  gab4_finish(a, gx, gy, min(4, a.xs - gx), w);
+  gab_pixels<1>(a, q, x0, y0);
 }
 
 // True when Weight()'s clamp of sad at 507 can change a weight that survives
@@ -2271,13 +2300,8 @@ __global__ void __launch_bounds__(256) k_filter(const __grid_constant__ FilterAr
 // (6.5) before the arithmetic.  The waits are bounded: on expiry the kernel
 // sets bit 8 of *err and stops waiting.
 // ---------------------------------------------------------------------------
-constexpr int kQW = 40, kQH = 34;                          // tile box (columns, rows)
 constexpr uint32_t kQBytes = 3u * kQH * kQW * 4u;          // one buffer, 16,320 bytes
 constexpr int kQWaitLimit = 1 << 22;
-
-struct __align__(128) QTile {
-  float s[3][kQH][kQW];
-};
 
 __device__ __forceinline__ bool q_wait(uint64_t* bar, uint32_t parity) {
   uint32_t done = 0;
@@ -2291,15 +2315,15 @@ __device__ __forceinline__ bool q_wait(uint64_t* bar, uint32_t parity) {
 
 // One landed tile of the TMA filter kernels: the mirrored ring outside the
 // image (rows first, then columns, so corners mirror twice; edge tiles are
-// the same for the whole CTA, which takes the barriers they need), then J.4
-// / K.5 / L.2 for 4 neighbouring pixels of a row per thread.
+// the same for the whole CTA, which takes the barriers they need), then its
+// pixels.
+template <int R>
 __device__ __forceinline__ void filter_tma_tile(const FilterArgs& a, QTile& q, int x0, int y0) {
   const int tid = threadIdx.x;
-  const int tx4 = tid & 7, ty = tid >> 3;   // pixels 4 tx4 .. 4 tx4 + 3 of row ty
   const bool top = y0 == 0, bottom = y0 + kGT + 1 > a.ys;
   const bool left = x0 == 0, right = x0 + kGT + 1 > a.xs;
   if (top || bottom) {
-    for (int k = tid; k < 2 * 3 * kQW; k += 256) {
+    for (int k = tid; k < 2 * 3 * kQW; k += 256 / R) {
       const int side = k / (3 * kQW), c = (k / kQW) % 3, lx = k % kQW;
       if (side == 0 && top) q.s[c][0][lx] = q.s[c][1][lx];
       if (side == 1 && bottom && a.ys - y0 + 1 < kQH)
@@ -2308,7 +2332,7 @@ __device__ __forceinline__ void filter_tma_tile(const FilterArgs& a, QTile& q, i
     __syncthreads();
   }
   if (left || right) {
-    for (int k = tid; k < 2 * 3 * kQH; k += 256) {
+    for (int k = tid; k < 2 * 3 * kQH; k += 256 / R) {
       const int side = k / (3 * kQH), c = (k / kQH) % 3, ly = k % kQH;
       if (side == 0 && left) q.s[c][ly][3] = q.s[c][ly][4];
       if (side == 1 && right && a.xs - x0 + 4 < kQW)
@@ -2316,22 +2340,7 @@ __device__ __forceinline__ void filter_tma_tile(const FilterArgs& a, QTile& q, i
     }
     __syncthreads();
   }
-  const int gx = x0 + 4 * tx4, gy = y0 + ty;
-  if (gx < a.xs && gy < a.ys) {
-    float w[3][3][6];   // image rows gy - 1 .. gy + 1, columns gx - 1 .. gx + 4
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-#pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        const float* row = &q.s[c][ty + r][4 * tx4 + 3];
-        const float4 m = *reinterpret_cast<const float4*>(row + 1);
-        w[c][r][0] = row[0];
-        w[c][r][1] = m.x; w[c][r][2] = m.y; w[c][r][3] = m.z; w[c][r][4] = m.w;
-        w[c][r][5] = row[5];
-      }
-    }
-    gab4_finish(a, gx, gy, min(4, a.xs - gx), w);
-  }
+  gab_pixels<R>(a, q, x0, y0);
 }
 
 // One 3-D TMA load of tile box {kQW, kQH, 3} at (x, y, 0) of tensor map tm into
@@ -2350,7 +2359,7 @@ __device__ __forceinline__ void tma_tile_load(const void* tm, int x, int y, uint
 // The pipeline of the TMA filter kernels over tiles blockIdx.x, + gridDim.x,
 // ... < ntiles: two buffers, "full" mbarriers (TMA transaction counts) and
 // "empty" ones (one arrival per warp); thread 0 loads the tile after next
-// into a buffer once the 8 warps released it.  src.issue(t, dst, bar) loads
+// into a buffer once its warps released it.  src.issue(t, dst, bar) loads
 // tile t (thread 0); src.consume(t, q) filters it (all threads).  A thread
 // whose bounded wait expires sets bit 8 of *err and skips every later wait
 // (and thread 0 every later load), following the same barriers as the
@@ -2415,6 +2424,7 @@ __device__ __forceinline__ void filter_tma_pipeline(Src& src, int ntiles, unsign
 }
 
 // Tiles of one image (ntx per row), its tensor map passed as a kernel parameter.
+template <int R>
 struct OneImageTiles {
   const FilterArgs& a;
   const CUtensorMap& tm;
@@ -2423,14 +2433,15 @@ struct OneImageTiles {
     tma_tile_load(&tm, (t % ntx) * kGT - 4, (t / ntx) * kGT - 1, dst, bar);
   }
   __device__ void consume(int t, QTile& q) const {
-    filter_tma_tile(a, q, (t % ntx) * kGT, (t / ntx) * kGT);
+    filter_tma_tile<R>(a, q, (t % ntx) * kGT, (t / ntx) * kGT);
   }
 };
 
-__global__ void __launch_bounds__(256) k_filter_tma(const __grid_constant__ FilterArgs a,
+template <int R>
+__global__ void __launch_bounds__(256 / R) k_filter_tma(const __grid_constant__ FilterArgs a,
                                                     const __grid_constant__ CUtensorMap tm,
                                                     int ntx, int ntiles, unsigned* err) {
-  OneImageTiles src{a, tm, ntx};
+  OneImageTiles<R> src{a, tm, ntx};
   filter_tma_pipeline(src, ntiles, err);
 }
 
@@ -2466,11 +2477,11 @@ struct BatchTiles {
     const FilterArgs& a = args[im];
     const int local = t - __ldg(prefix + im);
     const int tw = (a.xs + kGT - 1) / kGT;
-    filter_tma_tile(a, q, (local % tw) * kGT, (local / tw) * kGT);
+    filter_tma_tile<2>(a, q, (local % tw) * kGT, (local / tw) * kGT);
   }
 };
 
-__global__ void __launch_bounds__(256) k_filter_batch_tma(const FilterArgs* __restrict__ args,
+__global__ void __launch_bounds__(128) k_filter_batch_tma(const FilterArgs* __restrict__ args,
                                                           const int* __restrict__ prefix,
                                                           const CUtensorMap* __restrict__ maps,
                                                           int nimg, int total, unsigned* err) {
@@ -2951,7 +2962,7 @@ bool make_filter_tensor_map(const FilterArgs& a, void* tm) {
 
 void launch_filter_batch_tma(const FilterArgs* args, const int* prefix, const void* maps,
                              int nimg, int total, int grid, unsigned* err, cudaStream_t s) {
-  k_filter_batch_tma<<<grid < total ? grid : total, 256, 2 * sizeof(QTile), s>>>(
+  k_filter_batch_tma<<<grid < total ? grid : total, 128, 2 * sizeof(QTile), s>>>(
       args, prefix, static_cast<const CUtensorMap*>(maps), nimg, total, err);
 }
 
@@ -2995,7 +3006,7 @@ int batch_blocks_per_sm(int kind) {
   else if (kind == 2)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_filter_batch, 256, 0);
   else
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_filter_batch_tma, 256,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_filter_batch_tma, 128,
                                                       2 * sizeof(QTile));
   return e == cudaSuccess && n > 0 ? n : 1;
 }
@@ -3023,6 +3034,22 @@ void launch_epf_work(const FilterArgs& a, const int* list, const unsigned* count
   k<<<grid, 32, 0, s>>>(a, list, count, next);
 }
 
+// Resident CTAs of k_filter_tma<R> on the current device.
+template <int R>
+static int filter_tma_grid() {
+  static int grid_of[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  int& grid = grid_of[dev & 63];
+  if (grid == 0) {
+    int sms = 0, per = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_filter_tma<R>, 256 / R, 2 * sizeof(QTile));
+    grid = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
+  }
+  return grid;
+}
+
 void launch_filter(const FilterArgs& a, cudaStream_t s) {
   if (a.epf) {
     static const std::vector<int32_t> mul4 = [] {
@@ -3038,19 +3065,16 @@ void launch_filter(const FilterArgs& a, cudaStream_t s) {
   CUtensorMap tm;
   if (filter_tensor_map(a, &tm)) {
     // persistent grid of resident CTAs
-    static int grid_of[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    int& grid = grid_of[dev & 63];
-    if (grid == 0) {
-      int sms = 0, per = 0;
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_filter_tma, 256, 2 * sizeof(QTile));
-      grid = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
-    }
     const int ntx = (a.xs + kGT - 1) / kGT, ntiles = ntx * ((a.ys + kGT - 1) / kGT);
-    k_filter_tma<<<grid < ntiles ? grid : ntiles, 256, 2 * sizeof(QTile), s>>>(a, tm, ntx, ntiles,
-                                                                            a.err);
+    if (a.noise) {
+      const int grid = filter_tma_grid<1>();
+      k_filter_tma<1><<<grid < ntiles ? grid : ntiles, 256, 2 * sizeof(QTile), s>>>(a, tm, ntx,
+                                                                                 ntiles, a.err);
+    } else {
+      const int grid = filter_tma_grid<2>();
+      k_filter_tma<2><<<grid < ntiles ? grid : ntiles, 128, 2 * sizeof(QTile), s>>>(a, tm, ntx,
+                                                                                 ntiles, a.err);
+    }
     return;
   }
   dim3 grid((a.xs + kTW - 1) / kTW, (a.ys + kTH - 1) / kTH);
