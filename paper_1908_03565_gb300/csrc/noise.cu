@@ -2,11 +2,17 @@
 //
 // Per 256 x 256 group, eight generators run through the three channels
 // row by row, one step per 16-sample segment.  A thread owns one generator
-// for a chunk of 32 rows of one channel: it jumps its state to the chunk's
+// for a chunk of 8 rows of one channel: it jumps its state to the chunk's
 // first step with the GF(2) matrices of 2^b steps (the update is linear),
 // then steps through the chunk, writing samples 2i and 2i+1 of every
 // segment.  The jump replaces up to 12,288 dependent steps per generator by
 // at most 14 matrix-vector products, so the work spreads over all SMs.
+//
+// Bound by the chain of each generator (a step is about 25 dependent integer
+// instructions) and by having enough of them: chunks of 32 rows are 36 CTAs on
+// a 2047x1535 image, fewer than the SMs.  With J.3 and noise the request takes
+// 0.392 ms with chunks of 32 rows, 0.373 with 16, 0.360 with 8 and 0.365 with 4,
+// where the jumps (about 4,600 instructions each) outweigh the steps.
 #include <cuda_runtime.h>
 
 #include "internal.h"
@@ -19,7 +25,7 @@ namespace {
 __constant__ uint64_t c_njump[kNoiseJumpLevels * 256];
 
 constexpr int kGroup = 256;
-constexpr int kChunkRows = 32;
+constexpr int kChunkRows = 8;
 constexpr int kChunks = kGroup / kChunkRows;
 
 __device__ __forceinline__ uint64_t splitmix64(uint64_t z) {
