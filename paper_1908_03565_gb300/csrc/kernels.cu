@@ -40,7 +40,6 @@ namespace jxlr {
 __constant__ float c_llf[kLlfMaps * 256];
 __device__ float g_llf[kLlfMaps * 256];   // the same maps, read with per-lane addresses
 __constant__ float c_box[kLlfMaps * 256];
-__constant__ float c_odd[kOddFloats];
 __constant__ int32_t c_mul4[673];
 __constant__ float c_afv[256];
 __constant__ int c_dq_off[kNumCodes];
@@ -60,19 +59,23 @@ __device__ __forceinline__ int lg_w8(int code) { return (kW8Bits >> (2 * code)) 
 __device__ __forceinline__ int lg_h8(int code) { return (kH8Bits >> (2 * code)) & 3; }
 
 static void prefer_shared_carveout();
+template <int N>
+static bool odd_matches(const float* odd);   // odd_cos against the table
 
 bool upload_constants(const float* llf, const float* box, const float* odd,
                       const int32_t* mul4, const float* afv) {
   for (int c = 0; c < kNumCodes; ++c)   // the packed shape bits agree with the shape table
     if ((8 << ((kW8Bits >> (2 * c)) & 3)) != kShapeW[c] || (8 << ((kH8Bits >> (2 * c)) & 3)) != kShapeH[c])
       return false;
+  if (!odd_matches<32>(odd) || !odd_matches<16>(odd + 256) || !odd_matches<8>(odd + 320) ||
+      !odd_matches<4>(odd + 336) || !odd_matches<2>(odd + 340))
+    return false;
   prefer_shared_carveout();
   int offs[kNumCodes];
   for (int c = 0; c < kNumCodes; ++c) offs[c] = dequant_offset(c, 0);
   return cudaMemcpyToSymbol(c_llf, llf, sizeof(float) * kLlfMaps * 256) == cudaSuccess &&
          cudaMemcpyToSymbol(g_llf, llf, sizeof(float) * kLlfMaps * 256) == cudaSuccess &&
          cudaMemcpyToSymbol(c_box, box, sizeof(float) * kLlfMaps * 256) == cudaSuccess &&
-         cudaMemcpyToSymbol(c_odd, odd, sizeof(float) * kOddFloats) == cudaSuccess &&
          cudaMemcpyToSymbol(c_mul4, mul4, sizeof(int32_t) * 673) == cudaSuccess &&
          cudaMemcpyToSymbol(c_afv, afv, sizeof(float) * 256) == cudaSuccess &&
          cudaMemcpyToSymbol(c_dq_off, offs, sizeof(int) * kNumCodes) == cudaSuccess;
@@ -99,12 +102,40 @@ __device__ __forceinline__ int mirror_coord(int c, int size) {
   return c;
 }
 
-template <int N> struct OddOff;
-template <> struct OddOff<32> { static constexpr int v = 0; };
-template <> struct OddOff<16> { static constexpr int v = 256; };
-template <> struct OddOff<8> { static constexpr int v = 320; };
-template <> struct OddOff<4> { static constexpr int v = 336; };
-template <> struct OddOff<2> { static constexpr int v = 340; };
+// cos(k pi / 2N) for odd k < N, N = 32, 16, 8, 4, 2: the odd-part matrices of
+// the transforms (odd_tables) hold these values and their negatives.  As
+// literals they become immediate operands of the multiply-adds (from constant
+// memory they took a load into uniform registers each, 4% of the transform
+// kernel's instructions, and an eighth more code); upload_constants checks them
+// against the table.  With the conversions of coef_value and rcp_approx and the
+// map check in the transform kernel instead of a launch of its own: 4096^2 with
+// filters 0.581 -> 0.541 ms, without 0.250 -> 0.220, 1920x1088 0.122 -> 0.116.
+__device__ constexpr float kOddCos[31] = {
+    0x1.ff621ep-1f, 0x1.fa7558p-1f, 0x1.f0a7f0p-1f, 0x1.e21210p-1f, 0x1.ced7b0p-1f,
+    0x1.b72834p-1f, 0x1.9b3e04p-1f, 0x1.7b5df2p-1f, 0x1.57d694p-1f, 0x1.30ff80p-1f,
+    0x1.07387ap-1f, 0x1.b5d100p-2f, 0x1.58f9a8p-2f, 0x1.f19f98p-3f, 0x1.2c8106p-3f,
+    0x1.91f660p-5f, 0x1.fd88dap-1f, 0x1.e9f416p-1f, 0x1.c38b30p-1f, 0x1.8bc806p-1f,
+    0x1.44cf32p-1f, 0x1.e2b5d4p-2f, 0x1.294062p-2f, 0x1.917a6cp-4f, 0x1.f6297cp-1f,
+    0x1.a9b662p-1f, 0x1.1c73b4p-1f, 0x1.8f8b84p-3f, 0x1.d906bcp-1f, 0x1.87de2ap-2f,
+    0x1.6a09e6p-1f};
+// cos((2n + 1)(2j + 1) pi / 2N)
+template <int N>
+__host__ __device__ constexpr float odd_cos(int n, int j) {
+  int k = (2 * n + 1) * (2 * j + 1) % (4 * N);
+  if (k > 2 * N) k = 4 * N - k;
+  const bool neg = k > N;
+  if (neg) k = 2 * N - k;
+  const float v = kOddCos[32 - N + (k - 1) / 2];
+  return neg ? -v : v;
+}
+
+template <int N>
+static bool odd_matches(const float* odd) {
+  for (int n = 0; n < N / 2; ++n)
+    for (int j = 0; j < N / 2; ++j)
+      if (odd[n * (N / 2) + j] != odd_cos<N>(n, j)) return false;
+  return true;
+}
 
 // Unscaled N-point inverse DCT in registers (even/odd recursion).
 template <int N>
@@ -119,7 +150,7 @@ __device__ __forceinline__ void idct1d(float (&x)[N]) {
     for (int n = 0; n < H; ++n) {
       float s = 0.f;
 #pragma unroll
-      for (int j = 0; j < H; ++j) s = fmaf(x[2 * j + 1], c_odd[OddOff<N>::v + n * H + j], s);
+      for (int j = 0; j < H; ++j) s = fmaf(x[2 * j + 1], odd_cos<N>(n, j), s);
       o[n] = s;
     }
 #pragma unroll
@@ -603,7 +634,7 @@ __device__ __forceinline__ void fdct1d_raw(float (&x)[N]) {
     for (int j = 0; j < H; ++j) {
       float acc = 0.f;
 #pragma unroll
-      for (int n = 0; n < H; ++n) acc = fmaf(d[n], c_odd[OddOff<N>::v + n * H + j], acc);
+      for (int n = 0; n < H; ++n) acc = fmaf(d[n], odd_cos<N>(n, j), acc);
       x[2 * j + 1] = acc;
     }
 #pragma unroll
@@ -933,7 +964,7 @@ __device__ __forceinline__ void cell_map_entry(const uint8_t* __restrict__ vmap,
 __device__ void cell_setup(CellState& cs, const uint8_t* __restrict__ vmap,
                            const float* __restrict__ acmul, int gbx0, int gby0, int bw,
                            int bh, bool tc = false, const uint8_t* __restrict__ sharp = nullptr,
-                           const CellMap* pre = nullptr) {
+                           const CellMap* pre = nullptr, unsigned* status = nullptr) {
   const int tid = threadIdx.x;
   if (tid < 32) {
     const unsigned full = 0xffffffffu;
@@ -961,6 +992,20 @@ __device__ void cell_setup(CellState& cs, const uint8_t* __restrict__ vmap,
       ci = tc && tc_shape(code) ? 0 : col_items(code);
       fi = fwd_row_items(code);
       li = llf_items(code);
+    }
+    if (status) {
+      // C.5.4, the checks of k_validate on the cell's blocks: every varblock
+      // lies in one cell, so a map is a tiling when each cell is
+      const unsigned cov = __ballot_sync(full, tid < 16 && code == kCovered);
+      const unsigned in = __ballot_sync(full, tid < 16 && gbx0 + bx < bw && gby0 + by < bh);
+      const unsigned one = ((1u << w8) - 1u) << (4 * by + bx);
+      const unsigned foot = !valid ? 0u : one | (h8 > 1 ? one << 4 : 0u) |
+                                              (h8 > 2 ? one << 8 | one << 12 : 0u);
+      unsigned err = foot & ~(1u << b) & ~cov ? 8u : 0u;
+      if (tid < 16 && code != kCovered && !valid)
+        err |= code >= kNumCodes ? 1u : (bx % w8 || by % h8) ? 2u : 4u;
+      if (in & ~__reduce_or_sync(full, foot)) err |= 16u;
+      if (err) atomicOr(status, err);
     }
     const int key = valid ? code * 16 + b : 0x7fffffff;
     const bool lwork = valid && li > 0;
@@ -1237,6 +1282,24 @@ __device__ void tc_cell_pass(TcShared& ts, uint32_t& phase, unsigned* err, const
   }
 }
 
+// A quantised coefficient (j of the 8 in r) as a float: its 16 bits, offset by
+// 2^15, as the low bits of 2^23 + x (the conversion unit has an eighth of the
+// adders' rate).
+__device__ __forceinline__ float coef_value(const int4& r, int j) {
+  const uint32_t w = (j >> 1) == 0 ? r.x : (j >> 1) == 1 ? r.y : (j >> 1) == 2 ? r.z : r.w;
+  return __uint_as_float(__byte_perm(w ^ 0x80008000u, 0x4B000000u, (j & 1) ? 0x7632 : 0x7610)) -
+         8421376.f;
+}
+
+// 1 / q for an integer q of magnitude 2 .. 2^15 (no denormals on either side):
+// the reciprocal that __fdividef multiplies by, without its range handling
+// (0.145f * rcp_approx(q) has the bits of __fdividef(0.145f, q) for all of them).
+__device__ __forceinline__ float rcp_approx(float q) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(q));
+  return r;
+}
+
 // One 32x32 cell (cell coordinates cxi, cyi) of image a; 128 threads.
 // kDc: whether the DC-domain inputs (dc1, lfp) may be set (single-image
 // launches only).
@@ -1332,7 +1395,7 @@ __device__ __forceinline__ void recon_cell(const ReconArgs& a, int cxi, int cyi,
     *reinterpret_cast<float2*>(&slp[c][r][2 * q]) = v;
   }
   cell_setup(cs, a.vmap, a.acmul, gbx0, gby0, a.bw, a.bh, kTC, a.sigma ? a.sharp : nullptr,
-             kPf ? &cmap : nullptr);
+             kPf ? &cmap : nullptr, a.status);
   if (kTC) tc_fence_after();
 
   // ---- F.2 / F.3 / G: one 8-sample row chunk of all three channels -------
@@ -1350,9 +1413,8 @@ __device__ __forceinline__ void recon_cell(const ReconArgs& a, int cxi, int cyi,
       float q[3][8];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const int16_t* h = reinterpret_cast<const int16_t*>(&raw[c]);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) q[c][j] = static_cast<float>(h[j]);
+        for (int j = 0; j < 8; ++j) q[c][j] = coef_value(raw[c], j);
       }
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -1364,7 +1426,7 @@ __device__ __forceinline__ void recon_cell(const ReconArgs& a, int cxi, int cyi,
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const float qq = q[c][j];
-          const float adj = fabsf(qq) <= 1.f ? qq * omb : qq - __fdividef(0.145f, qq);
+          const float adj = fabsf(qq) <= 1.f ? qq * omb : __fsub_rn(qq, __fmul_rn(0.145f, rcp_approx(qq)));
           out[c][j] = adj * v.acmul * mm[j];
         }
       }

@@ -66,6 +66,8 @@ struct ReconArgs {
   const float* dc1;           // [3][bh][bw] DC after F.2 smoothing and G, or nullptr
   const float* lfp;           // [3][2bh][2bw] Annex H coefficients, or nullptr
   EpfSink epf;                // with sigma
+  unsigned* status;           // C.5.4: the flags of an ill-formed map are set here (as by
+                              // launch_validate), or nullptr: not checked
 };
 
 struct SigmaArgs {
