@@ -107,7 +107,7 @@ __device__ __forceinline__ int mirror_coord(int c, int size) {
 // literals they become immediate operands of the multiply-adds (from constant
 // memory they took a load into uniform registers each, 4% of the transform
 // kernel's instructions, and an eighth more code); upload_constants checks them
-// against the table.  With the conversions of coef_value and rcp_approx and the
+// against the table.  With the conversions of coef_pair and rcp_approx and the
 // map check in the transform kernel instead of a launch of its own: 4096^2 with
 // filters 0.581 -> 0.541 ms, without 0.250 -> 0.220, 1920x1088 0.122 -> 0.116.
 __device__ constexpr float kOddCos[31] = {
@@ -1282,18 +1282,19 @@ __device__ void tc_cell_pass(TcShared& ts, uint32_t& phase, unsigned* err, const
   }
 }
 
-// A quantised coefficient (j of the 8 in r) as a float: its 16 bits, offset by
-// 2^15, as the low bits of 2^23 + x (the conversion unit has an eighth of the
-// adders' rate).
-__device__ __forceinline__ float coef_value(const int4& r, int j) {
-  const uint32_t w = (j >> 1) == 0 ? r.x : (j >> 1) == 1 ? r.y : (j >> 1) == 2 ? r.z : r.w;
-  return __uint_as_float(__byte_perm(w ^ 0x80008000u, 0x4B000000u, (j & 1) ? 0x7632 : 0x7610)) -
-         8421376.f;
+// Quantised coefficients 2 i and 2 i + 1 of the 8 in r as floats: the 16 bits
+// of each, offset by 2^15, as the low bits of 2^23 + x (the conversion unit has
+// an eighth of the adders' rate).
+__device__ __forceinline__ float2 coef_pair(const int4& r, int i) {
+  const uint32_t w = (i == 0 ? r.x : i == 1 ? r.y : i == 2 ? r.z : r.w) ^ 0x80008000u;
+  return __fadd2_rn(make_float2(__uint_as_float(__byte_perm(w, 0x4B000000u, 0x7610)),
+                                __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7632))),
+                    f2(-8421376.f));
 }
 
 // 1 / q for an integer q of magnitude 2 .. 2^15 (no denormals on either side):
-// the reciprocal that __fdividef multiplies by, without its range handling
-// (0.145f * rcp_approx(q) has the bits of __fdividef(0.145f, q) for all of them).
+// the documented approximate reciprocal.  0.145f * rcp_approx(q) was compared
+// with the quotient of the two by CUDA's fast division for all of these q.
 __device__ __forceinline__ float rcp_approx(float q) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(q));
@@ -1410,48 +1411,70 @@ __device__ __forceinline__ void recon_cell(const ReconArgs& a, int cxi, int cyi,
       const int cxl = W >> 3, cyl = H >> 3;
       const int tile = (gy >> 6) * a.tw + (gx >> 6);
       const float kx = a.cfl[2 * tile], kb = a.cfl[2 * tile + 1];
-      float q[3][8];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) q[c][j] = coef_value(raw[c], j);
-      }
+      // two neighbouring coefficients per paired operation (this and the tests
+      // left out below: 4096^2 without filters 0.231 -> 0.219 ms, 8192^2 u8 with
+      // them 1.952 -> 1.908, same bits)
+      float2 o2[3][4];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const float* m = a.dequant + v.dqoff + ((c * H + vv) << v.lw) + u0;
         const float4 m0 = __ldg(reinterpret_cast<const float4*>(m));
         const float4 m1 = __ldg(reinterpret_cast<const float4*>(m + 4));
-        const float mm[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
-        const float omb = a.one_minus_bias[c];
+        const float2 mm[4] = {make_float2(m0.x, m0.y), make_float2(m0.z, m0.w),
+                              make_float2(m1.x, m1.y), make_float2(m1.z, m1.w)};
+        const float2 omb = f2(a.one_minus_bias[c]);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const float qq = q[c][j];
-          const float adj = fabsf(qq) <= 1.f ? qq * omb : __fsub_rn(qq, __fmul_rn(0.145f, rcp_approx(qq)));
-          out[c][j] = adj * v.acmul * mm[j];
+        for (int i = 0; i < 4; ++i) {
+          const float2 q = coef_pair(raw[c], i);
+          const float2 one = __fmul2_rn(q, omb);
+          const float2 far = __fadd2_rn(
+              q, __fmul2_rn(f2(-0.145f), make_float2(rcp_approx(q.x), rcp_approx(q.y))));
+          const float2 adj = make_float2(fabsf(q.x) <= 1.f ? one.x : far.x,
+                                         fabsf(q.y) <= 1.f ? one.y : far.y);
+          o2[c][i] = __fmul2_rn(__fmul2_rn(adj, f2(v.acmul)), mm[i]);
         }
       }
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const bool llf = (u0 + j) < cxl && vv < cyl;
-        if (llf) {
-          if (kDc && a.dc1) {   // F.2 smoothing and G already applied per block
+      for (int i = 0; i < 4; ++i) {
+        o2[0][i] = __ffma2_rn(f2(kx), o2[1][i], o2[0][i]);
+        o2[2][i] = __ffma2_rn(f2(kb), o2[1][i], o2[2][i]);
+      }
 #pragma unroll
-            for (int c = 0; c < 3; ++c) out[c][j] = sdc[c][v.by + vv][v.bx + u0 + j];
-          } else {
-            const float dx = a.m_dc[0] * q[0][j], dy = a.m_dc[1] * q[1][j],
-                        db = a.m_dc[2] * q[2][j];
-            out[0][j] = fmaf(a.kx_dc, dy, dx);
-            out[1][j] = dy;
-            out[2][j] = fmaf(a.kb_dc, dy, db);
-          }
-        } else {
-          out[0][j] = fmaf(kx, out[1][j], out[0][j]);
-          out[2][j] = fmaf(kb, out[1][j], out[2][j]);
-          if (kDc && a.lfp && (u0 + j) < 2 * cxl && vv < 2 * cyl) {   // Annex H prediction
+      for (int c = 0; c < 3; ++c)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) out[c][j] += slp[c][2 * v.by + vv][2 * v.bx + u0 + j];
+        for (int i = 0; i < 4; ++i) { out[c][2 * i] = o2[c][i].x; out[c][2 * i + 1] = o2[c][i].y; }
+      // A varblock's LLF slots (at most 4 x 4) lie in its first chunk of a row,
+      // and so do the slots of Annex H (at most 8 x 8): the other chunks need no
+      // test per coefficient.
+      if (kDc && a.lfp && u0 == 0 && vv < 2 * cyl) {   // Annex H prediction
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (j < 2 * cxl) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) out[c][j] += slp[c][2 * v.by + vv][2 * v.bx + j];
           }
-        }
+      }
+      if (u0 == 0 && vv < cyl) {
+        float2 d2[3][2];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) d2[c][i] = coef_pair(raw[c], i);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j < cxl) {
+            if (kDc && a.dc1) {   // F.2 smoothing and G already applied per block
+#pragma unroll
+              for (int c = 0; c < 3; ++c) out[c][j] = sdc[c][v.by + vv][v.bx + j];
+            } else {
+              const float dx = a.m_dc[0] * ((j & 1) ? d2[0][j >> 1].y : d2[0][j >> 1].x);
+              const float dy = a.m_dc[1] * ((j & 1) ? d2[1][j >> 1].y : d2[1][j >> 1].x);
+              const float db = a.m_dc[2] * ((j & 1) ? d2[2][j >> 1].y : d2[2][j >> 1].x);
+              out[0][j] = fmaf(a.kx_dc, dy, dx);
+              out[1][j] = dy;
+              out[2][j] = fmaf(a.kb_dc, dy, db);
+            }
+          }
       }
     } else {
 #pragma unroll
