@@ -829,7 +829,12 @@ __device__ void cell_sigma(float (*S)[kPR][kRS], CellState& cs, const SigmaParam
       const float4 v1 = *reinterpret_cast<const float4*>(&S[c][ly][lx0 + 4]);
       float g[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
 #pragma unroll
-      for (int j = 0; j < 8; ++j) g[j] = guide_scaled(sp, c, g[j]);
+      for (int j = 0; j < 8; j += 2) {   // guide_scaled of two samples
+        const float2 t = __fmul2_rn(__fadd2_rn(make_float2(g[j], g[j + 1]), f2(-sp.gmin[c])),
+                                    f2(sp.gscale[c]));
+        g[j] = t.x;
+        g[j + 1] = t.y;
+      }
       if (store) {
         uint2 w;
         w.x = pack4(guide_byte(g[0]), guide_byte(g[1]), guide_byte(g[2]), guide_byte(g[3]));
@@ -907,20 +912,26 @@ __device__ void cell_sigma(float (*S)[kPR][kRS], CellState& cs, const SigmaParam
     __syncthreads();
     pm = s_pass;
   }
-  // planar XYB [3][hp][wp] (xyb_out) and the unchanged blocks' copy, float4
-  // per thread step
+  // planar XYB [3][hp][wp] (xyb_out) and the unchanged blocks' copy: a thread
+  // has float4 k4 of rows y and y + 16, a plane's offset apart per channel (with
+  // a division into channel, row and column per float4 and the guide unpaired,
+  // the 48-image batch took 0.719 instead of 0.706 ms, 8192^2 1.902 / 1.884)
   if (pm || xyb_out) {
-    const int hp = 8 * bh, wp = 8 * bw;
-    for (int i = tid; i < 3 * 32 * 8; i += blockDim.x) {
-      const int c = i / 256, y = (i >> 3) & 31, k4 = i & 7;
+    const int hp = 8 * bh, wp = 8 * bw, k4 = tid & 7;
+    const int gx = gbx0 * 8 + 4 * k4;
+    const size_t plane = static_cast<size_t>(hp) * wp;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int y = (tid >> 3) + 16 * h, gy = gby0 * 8 + y;
       const bool pass = (pm >> ((y >> 3) * 4 + (k4 >> 1))) & 1u;
-      if (!pass && !xyb_out) continue;
-      const int gy = gby0 * 8 + y, gx = gbx0 * 8 + 4 * k4;
-      if (gy < hp && gx < wp) {
+      if (gy >= hp || gx >= wp || (!pass && !xyb_out)) continue;
+      float* const xo = xyb_out + static_cast<size_t>(gy) * wp + gx;
+      float* const po = epf.pass + static_cast<size_t>(gy) * epf.prs + gx;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
         const float4 v4 = *reinterpret_cast<const float4*>(&S[c][y][4 * k4]);
-        if (xyb_out) *reinterpret_cast<float4*>(xyb_out + (static_cast<size_t>(c) * hp + gy) * wp + gx) = v4;
-        if (pass)
-          *reinterpret_cast<float4*>(epf.pass + c * epf.pps + static_cast<size_t>(gy) * epf.prs + gx) = v4;
+        if (xyb_out) *reinterpret_cast<float4*>(xo + c * plane) = v4;
+        if (pass) *reinterpret_cast<float4*>(po + c * epf.pps) = v4;
       }
     }
   }
