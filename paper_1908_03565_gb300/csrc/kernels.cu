@@ -409,8 +409,12 @@ struct CellState {
   CellVB vb[16];
   int nvb;
   int owner[16];         // per in-cell block: index into vb, or -1
-  int row_pre[17];       // prefix sums of row-phase items
-  int col_pre[17];       // prefix sums of column-phase items
+  // The varblock of each row- and column-phase item (a varblock's items are a
+  // multiple of 12 in the row phase, of 24 in the column phase): code | bx << 4
+  // | by << 6 | (its first item / 12 or / 24) << 8.  A table instead of a search
+  // through prefix sums: 8192^2 u8 1.871 -> 1.861 ms, same bits.
+  uint16_t row_of[32], col_of[16];
+  int row_total, col_total;
   int frow_pre[17];      // prefix sums of the forward row-phase items (J.3)
   // LLF phase (I.2.7 and the DC pre-steps of DCT4 / 8x4 / 4x8): the
   // varblocks with such work in order of decreasing LLF size n, each with
@@ -452,6 +456,18 @@ __device__ __forceinline__ int llf_items(int code) {
 }
 
 __device__ __forceinline__ int col_items(int code) { return 3 * (8 << lg_w8(code)); }
+
+// Item it of the row (kUnit 12) or column (24) phase: its varblock's code, place
+// and shape, and its number k among the varblock's items.
+template <int kUnit>
+__device__ __forceinline__ CellVB item_of(const uint16_t* of, int it, int& k) {
+  const unsigned e = of[static_cast<unsigned>(it) / kUnit];
+  CellVB v;
+  v.code = e & 15; v.bx = (e >> 4) & 3; v.by = (e >> 6) & 3;
+  v.lw = 3 + lg_w8(v.code); v.lh = 3 + lg_h8(v.code);
+  k = it - kUnit * static_cast<int>(e >> 8);
+  return v;
+}
 
 // One AuxIDCT2x2 level of I.2.4.2 on the top-left 2h x 2h of q, in place:
 // the 2x2 groups at (y, x), (y, h + x), (h + y, x), (h + y, h + x) become
@@ -1038,6 +1054,7 @@ __device__ void cell_setup(CellState& cs, const uint8_t* __restrict__ vmap,
     const int pr = before & 1023u, pc = (before >> 10) & 1023u, pf = before >> 20;
     const int n = __popc(__ballot_sync(full, valid));
     const int nl = __popc(__ballot_sync(full, lwork));
+    const unsigned sum = __reduce_add_sync(full, valid ? w1 : 0u);
     if (tid < 16) {
       cs.owner[tid] = -1;
       cs.bacmul[tid] = am;
@@ -1046,7 +1063,9 @@ __device__ void cell_setup(CellState& cs, const uint8_t* __restrict__ vmap,
     if (tid == 0) {
       cs.nvb = n;
       cs.nllf = nl;
-      cs.row_pre[0] = cs.col_pre[0] = cs.frow_pre[0] = cs.llf_pre[0] = 0;
+      cs.frow_pre[0] = cs.llf_pre[0] = 0;
+      cs.row_total = sum & 1023u;
+      cs.col_total = (sum >> 10) & 1023u;
     }
     __syncwarp();
     if (valid) {
@@ -1056,8 +1075,11 @@ __device__ void cell_setup(CellState& cs, const uint8_t* __restrict__ vmap,
       v.dqoff = c_dq_off[code];
       v.pad = 0;
       cs.vb[rank] = v;
-      cs.row_pre[rank + 1] = pr + ri;
-      cs.col_pre[rank + 1] = pc + ci;
+      const unsigned place = code | bx << 4 | by << 6;
+      for (int i = pr / 12; i < (pr + ri) / 12; ++i)
+        cs.row_of[i] = static_cast<uint16_t>(place | (pr / 12) << 8);
+      for (int i = pc / 24; i < (pc + ci) / 24; ++i)
+        cs.col_of[i] = static_cast<uint16_t>(place | (pc / 24) << 8);
       cs.frow_pre[rank + 1] = pf + fi;
       if (lwork) {
         cs.llf_vb[lrank] = rank;
@@ -1563,21 +1585,19 @@ __device__ __forceinline__ void recon_cell(const ReconArgs& a, int cxi, int cyi,
 
   // ---- I.2.4 row pass ------------------------------------------------------
   {
-    const int total = cs.row_pre[cs.nvb];
-    int vi = 0;
-    for (int it = tid; it < total; it += blockDim.x) {
-      while (it >= cs.row_pre[vi + 1]) ++vi;
-      row_item(S, T, cs.vb[vi], it - cs.row_pre[vi]);
+    for (int it = tid; it < cs.row_total; it += blockDim.x) {
+      int k;
+      const CellVB v = item_of<12>(cs.row_of, it, k);
+      row_item(S, T, v, k);
     }
   }
   __syncthreads();
   // ---- column pass ---------------------------------------------------------
   {
-    const int total = cs.col_pre[cs.nvb];
-    int vi = 0;
-    for (int it = tid; it < total; it += blockDim.x) {
-      while (it >= cs.col_pre[vi + 1]) ++vi;
-      col_item(S, T, cs.vb[vi], it - cs.col_pre[vi]);
+    for (int it = tid; it < cs.col_total; it += blockDim.x) {
+      int k;
+      const CellVB v = item_of<24>(cs.col_of, it, k);
+      col_item(S, T, v, k);
     }
   }
   __syncthreads();
@@ -1774,11 +1794,10 @@ __global__ void __launch_bounds__(128, 6) k_qco(const __grid_constant__ QcoArgs 
   }
   __syncthreads();
   {
-    const int total = cs.col_pre[cs.nvb];
-    int vi = 0;
-    for (int it = tid; it < total; it += blockDim.x) {
-      while (it >= cs.col_pre[vi + 1]) ++vi;
-      fwd_col_item(S, T, cs.vb[vi], it - cs.col_pre[vi]);
+    for (int it = tid; it < cs.col_total; it += blockDim.x) {
+      int k;
+      const CellVB v = item_of<24>(cs.col_of, it, k);
+      fwd_col_item(S, T, v, k);
     }
   }
   __syncthreads();
@@ -1884,20 +1903,18 @@ __global__ void __launch_bounds__(128, 6) k_qco(const __grid_constant__ QcoArgs 
   }
   __syncthreads();
   {
-    const int total = cs.row_pre[cs.nvb];
-    int vi = 0;
-    for (int it = tid; it < total; it += blockDim.x) {
-      while (it >= cs.row_pre[vi + 1]) ++vi;
-      row_item(S, T, cs.vb[vi], it - cs.row_pre[vi]);
+    for (int it = tid; it < cs.row_total; it += blockDim.x) {
+      int k;
+      const CellVB v = item_of<12>(cs.row_of, it, k);
+      row_item(S, T, v, k);
     }
   }
   __syncthreads();
   {
-    const int total = cs.col_pre[cs.nvb];
-    int vi = 0;
-    for (int it = tid; it < total; it += blockDim.x) {
-      while (it >= cs.col_pre[vi + 1]) ++vi;
-      col_item(S, T, cs.vb[vi], it - cs.col_pre[vi]);
+    for (int it = tid; it < cs.col_total; it += blockDim.x) {
+      int k;
+      const CellVB v = item_of<24>(cs.col_of, it, k);
+      col_item(S, T, v, k);
     }
   }
   __syncthreads();
