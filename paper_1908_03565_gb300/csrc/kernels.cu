@@ -412,8 +412,11 @@ struct CellState {
   // The varblock of each row- and column-phase item (a varblock's items are a
   // multiple of 12 in the row phase, of 24 in the column phase): code | bx << 4
   // | by << 6 | (its first item / 12 or / 24) << 8.  A table instead of a search
-  // through prefix sums: 8192^2 u8 1.871 -> 1.861 ms, same bits.
-  uint16_t row_of[32], col_of[16];
+  // through prefix sums: 8192^2 u8 1.871 -> 1.861 ms, same bits.  A tiling has at
+  // most 384 items of either kind; a map that is not one (refused, but the cell
+  // runs) at most 768: 4 varblocks of height 4 from row 0, 4 of height 2 from row
+  // 2 and 8 of height 1, overlapping (columns likewise).
+  uint16_t row_of[64], col_of[32];
   int row_total, col_total;
   int frow_pre[17];      // prefix sums of the forward row-phase items (J.3)
   // LLF phase (I.2.7 and the DC pre-steps of DCT4 / 8x4 / 4x8): the
@@ -1036,8 +1039,8 @@ __device__ void cell_setup(CellState& cs, const uint8_t* __restrict__ vmap,
     }
     // the order and the item counts of all 16 blocks by two shuffles a block
     // (six: 8192^2 u8 1.908 instead of 1.902 ms; the other warps wait here):
-    // word 0 key (8 bits) | LLF key (8) | LLF items, word 1 row | column (10) |
-    // forward row items (10 each; the sums over a cell are at most 384)
+    // word 0 key (8 bits) | LLF key (8) | LLF items, word 1 row | column |
+    // forward row items (10 each; the sums over a cell are at most 768)
     const bool lwork = valid && li > 0;
     const unsigned key = valid ? code * 16 + b : 255;
     const unsigned lkey = lwork ? (4 - lg_w8(code) - lg_h8(code)) * 16 + b : 255;
