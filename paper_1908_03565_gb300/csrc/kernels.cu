@@ -34,6 +34,7 @@
 
 #include "internal.h"
 #include "kernels.h"
+#include "launch.h"
 
 namespace jxlr {
 
@@ -1605,6 +1606,9 @@ __device__ __forceinline__ void recon_cell(const ReconArgs& a, int cxi, int cyi,
   }
   __syncthreads();
 
+  // the next kernel's blocks may take the places of finished ones from here on
+  // (not from the start: they would hold places that other streams' kernels want)
+  if (!kPf && !kTC) let_next_start();
   // ---- output ---------------------------------------------------------------
   // (persistent form: T is free from here on; the next cell's coefficients
   // and map entries arrive during the stores)
@@ -2499,6 +2503,7 @@ __device__ __forceinline__ void filter_tma_pipeline(Src& src, int ntiles, unsign
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  if (Src::kAfter) wait_for_stream();   // every read of the tiles is a TMA load after this
   int t = blockIdx.x;
   const int G = static_cast<int>(gridDim.x);
   // thread 0: the use of buffer 0 / 1 whose load it has not seen land (-1: none)
@@ -2545,6 +2550,7 @@ __device__ __forceinline__ void filter_tma_pipeline(Src& src, int ntiles, unsign
 // Tiles of one image (ntx per row), its tensor map passed as a kernel parameter.
 template <int R>
 struct OneImageTiles {
+  static constexpr bool kAfter = R == 2;   // launched by launch_after
   const FilterArgs& a;
   const CUtensorMap& tm;
   int ntx;
@@ -2569,6 +2575,7 @@ __global__ void __launch_bounds__(256 / R) k_filter_tma(const __grid_constant__ 
 // The tiles a CTA visits only increase, so each of the two streams (loads
 // issued by thread 0, tiles consumed) keeps its own image cursor.
 struct BatchTiles {
+  static constexpr bool kAfter = false;
   const FilterArgs* args;
   const int* prefix;
   const CUtensorMap* maps;
@@ -2970,8 +2977,9 @@ __global__ void __launch_bounds__(32, 16) k_epf_work(const __grid_constant__ Fil
                                                      const unsigned* __restrict__ count,
                                                      unsigned* next) {
   bool needed = false;
-  epf_work_groups<kClamp, kPlane>(a, list, static_cast<int>(*count), blockIdx.x, gridDim.x, needed,
-                                  next);
+  const unsigned zero = wait_for_stream();
+  epf_work_groups<kClamp, kPlane>(a, list + zero, static_cast<int>(count[zero]), blockIdx.x,
+                                  gridDim.x, needed, next);
 }
 
 // Multi-image form: the groups of 2 listed blocks of all images, image after
@@ -3150,7 +3158,7 @@ void launch_epf_work(const FilterArgs& a, const int* list, const unsigned* count
   const bool clamp = filter_needs_clamp(a), plane = a.guide != nullptr;
   auto* k = clamp ? (plane ? k_epf_work<true, true> : k_epf_work<true, false>)
                   : (plane ? k_epf_work<false, true> : k_epf_work<false, false>);
-  k<<<grid, 32, 0, s>>>(a, list, count, next);
+  launch_after(k, grid, 32, 0, s, a, list, count, next);
 }
 
 // Resident CTAs of k_filter_tma<R> on the current device.
@@ -3191,8 +3199,8 @@ void launch_filter(const FilterArgs& a, cudaStream_t s) {
                                                                                  ntiles, a.err);
     } else {
       const int grid = filter_tma_grid<2>();
-      k_filter_tma<2><<<grid < ntiles ? grid : ntiles, 128, 2 * sizeof(QTile), s>>>(a, tm, ntx,
-                                                                                 ntiles, a.err);
+      launch_after(k_filter_tma<2>, grid < ntiles ? grid : ntiles, 128, 2 * sizeof(QTile), s, a, tm,
+                   ntx, ntiles, a.err);
     }
     return;
   }
