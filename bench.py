@@ -45,12 +45,12 @@ EPF_OPS_PER_FILTERED_PX = 56 * 8 + 4 + 4
 GUIDE_OPS_PER_PX = 17
 # DRAM bytes (read + write) of one k_epf_work launch, from an ncu capture of
 # the current kernel on the same statistics at 4096x2048 (50,730 listed
-# blocks): 99,106,048 + 23,353,856; scaled to a launch by its pixels.  Set to
+# blocks): 102,867,200 + 19,798,784; scaled to a launch by its pixels.  Set to
 # None whenever the kernel changes until it is captured again.
-EPF_WORK_DRAM_BYTES_4096x2048 = 99106048 + 23353856
+EPF_WORK_DRAM_BYTES_4096x2048 = 102867200 + 19798784
 # The same for one k_recon launch (4096x2048, EPF + Gaborish: coefficients
-# in, XYB and the copy of the blocks J.2 leaves unchanged out).
-RECON_DRAM_BYTES_4096x2048 = 51271680 + 119876096
+# in, XYB, guide bytes and the copy of the blocks J.2 leaves unchanged out).
+RECON_DRAM_BYTES_4096x2048 = 51312384 + 136635392
 CPU_SAMPLE = 1024         # oracle sample on one core: one 1024x1024 image, same statistics
 CPU_SAMPLE_ALL = 2048     # oracle sample on every host core: one 2048x2048 image
 
