@@ -1664,6 +1664,7 @@ __device__ __forceinline__ void recon_cell(const ReconArgs& a, int cxi, int cyi,
 }
 
 __global__ void __launch_bounds__(128, 7) k_recon(const __grid_constant__ ReconArgs a) {
+  if (a.dc1) wait_for_stream();   // the DC and Annex H kernels, where they come before
   recon_cell(a, blockIdx.x, blockIdx.y);
 }
 
@@ -1730,7 +1731,9 @@ void launch_recon(const ReconArgs& a, cudaStream_t s, int variant) {
     k_recon_pf<<<grid < ncells ? grid : ncells, 128, 0, s>>>(a, ncx, ncells);
     return;
   }
-  k_recon<<<dim3(ncx, ncy), 128, 0, s>>>(a);
+  // behind the DC kernels it starts while they end
+  if (a.dc1) launch_after(k_recon, dim3(ncx, ncy), dim3(128), 0, s, a);
+  else k_recon<<<dim3(ncx, ncy), 128, 0, s>>>(a);
 }
 
 void launch_recon_batch(const ReconArgs* args, const int* item_cell, int total, int grid,

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "launch.h"
 #include "lf.h"
 
 namespace jxlr {
@@ -79,6 +80,7 @@ __global__ void __launch_bounds__(64) k_dc_cell(const __grid_constant__ LfArgs a
   __shared__ uint8_t own[4][4];
   __shared__ uint8_t sv[12][12];          // map of the 3 x 3 cells around this one
   __shared__ float s_up[kLfUpFloats];
+  let_next_start();
   const int tid = threadIdx.x;
   const int cbx = 4 * blockIdx.x, cby = 4 * blockIdx.y;
   const int ox = cbx - 4, oy = cby - 4;
@@ -182,7 +184,9 @@ __global__ void __launch_bounds__(128) k_lf_cell(const __grid_constant__ LfArgs 
   __shared__ float Us[3][8][8];
   __shared__ float s_inv[kLfInvFloats];
   const int tid = threadIdx.x;
+  let_next_start();
   if (tid < kLfInvFloats) s_inv[tid] = c_lf_inv[tid];
+  wait_for_stream();   // k_dc_cell's planes
   const int X0 = 8 * blockIdx.x, Y0 = 8 * blockIdx.y;     // cell origin in DC2x2 samples
   const int pw = 2 * a.bw, ph = 2 * a.bh;
   const int gx0 = X0 & ~63, gy0 = Y0 & ~63;
@@ -275,7 +279,7 @@ int launch_lf(const LfArgs& a, cudaStream_t s) {
   const dim3 cells((a.bw + 3) / 4, (a.bh + 3) / 4);
   k_dc_cell<<<cells, 64, 0, s>>>(a);
   if (!a.predict) return 1;
-  k_lf_cell<<<cells, 128, 0, s>>>(a);
+  launch_after(k_lf_cell, cells, dim3(128), 0, s, a);
   return 2;
 }
 

@@ -12,11 +12,12 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("xs,ys", [(1, 1), (48, 40), (131, 77), (1024, 520)])
 @pytest.mark.parametrize("epf", [0, 1])
-def test_back_to_back(gpu_lib, xs, ys, epf):
+@pytest.mark.parametrize("dc", [0, 1, 2])     # none; F.2; F.2 and Annex H
+def test_back_to_back(gpu_lib, xs, ys, epf, dc):
     import torch
     imgs = [synth.make_image(xs, ys, 3, coef_scale=2.0, acmul=0.5, dc='smooth'),
             synth.make_image(xs, ys, 4), synth.make_image(xs, ys, 5, dc='smooth')]
-    p = binding.filter_defaults(epf=epf, gab=1)
+    p = binding.filter_defaults(epf=epf, gab=1, dc_smooth=dc > 0, lf_predict=dc > 1)
     dev = [binding.to_device(i, torch) for i in imgs]
     new = lambda: torch.full((ys, xs, 3), 7, dtype=torch.float32, device="cuda")
     with binding.Context(device=0) as ctx:
@@ -27,7 +28,7 @@ def test_back_to_back(gpu_lib, xs, ys, epf):
             ctx.poll(ctx.submit(dev[k % 3], p, o, binding.OUT_F32_LINEAR, True))
     for k, o in enumerate(outs):
         assert np.array_equal(o.cpu().numpy().view(np.uint32), want[k % 3].view(np.uint32))
-    if epf:
+    if epf and not dc:
         for d, w in zip(dev, want):
             o = new()
             torch.cuda.synchronize()
