@@ -1026,7 +1026,13 @@ __device__ void cell_setup(CellState& cs, const uint8_t* __restrict__ vmap,
     }
     if (status) {
       // C.5.4, the checks of k_validate on the cell's blocks: every varblock
-      // lies in one cell, so a map is a tiling when each cell is
+      // lies in one cell, so a map is a tiling when each cell is.  A cell is
+      // one when its footprints hold n blocks in all, n the number of its
+      // blocks, and add up, as numbers, to the mask of those blocks: no fewer
+      // than n powers of two add up to a number of n set bits, and n of them
+      // only as its bits, each once.  (Their union alone misses two varblocks
+      // that cross on a block coded as covered.)  One sum holds both: at most
+      // 16 masks of 16 bits below bit 20, at most 256 blocks above.
       const unsigned cov = __ballot_sync(full, tid < 16 && code == kCovered);
       const unsigned in = __ballot_sync(full, tid < 16 && gbx0 + bx < bw && gby0 + by < bh);
       const unsigned one = ((1u << w8) - 1u) << (4 * by + bx);
@@ -1035,7 +1041,8 @@ __device__ void cell_setup(CellState& cs, const uint8_t* __restrict__ vmap,
       unsigned err = foot & ~(1u << b) & ~cov ? 8u : 0u;
       if (tid < 16 && code != kCovered && !valid)
         err |= code >= kNumCodes ? 1u : (bx % w8 || by % h8) ? 2u : 4u;
-      if (in & ~__reduce_or_sync(full, foot)) err |= 16u;
+      if (__reduce_add_sync(full, foot | __popc(foot) << 20) != (in | __popc(in) << 20))
+        err |= 16u;
       if (err) atomicOr(status, err);
     }
     // the order and the item counts of all 16 blocks by two shuffles a block
