@@ -79,7 +79,12 @@ typedef enum {
 typedef struct {
   int device;              /* CUDA device ordinal                             */
   size_t hbm_cap_bytes;    /* device bytes the context may hold for request
-                              scratch and staged inputs; 0 = no cap           */
+                              scratch and staged inputs; 0 = no cap.  With
+                              several slots a cap admits what the filters' own
+                              scratch allows (24 bytes a pixel with the EPF);
+                              the 3 bytes a pixel of guide bytes that speed the
+                              EPF up are then kept only in room that a slot's
+                              scratch already has                             */
   int max_slots;           /* requests in flight at once (>= 1); each slot
                               owns one CUDA stream and its scratch arena      */
   int precision;           /* a jxlr_precision                                */

@@ -379,19 +379,25 @@ jxlr_status acquire_slot(jxl_recon_ctx* ctx, size_t need, uint64_t pixels, Slot*
   return JXLR_OK;
 }
 
-// acquire_slot() for a request with the EPF: its arena has room for the J.2.2
-// guide bytes behind `need` when the request with them fits under the HBM cap
-// and on the device (*plane), else the request runs without that plane (the
-// J.2 kernel then forms the bytes from the samples), so that it needs no more
-// memory than the filter itself.
+// acquire_slot() for a request with the EPF, which can use room for the J.2.2
+// guide bytes behind `need` (*plane: it has it); without, the J.2 kernel forms
+// the bytes from the samples (0.645 instead of 0.602 ms at 4096^2).  With no
+// cap, or with one slot, whose request leaves room for no other, the plane is
+// asked for with the rest and left out where that does not fit.  With several
+// slots under a cap it may cost no request its place, of the later ones
+// neither: the arena is the one that `need` alone asks for, and the plane is
+// used where that has room.
 jxlr_status acquire_epf_slot(jxl_recon_ctx* ctx, size_t need, size_t plane_bytes, uint64_t pixels,
                              Slot** out, bool* plane) {
   *plane = plane_bytes != 0;
-  jxlr_status st = acquire_slot(ctx, need + plane_bytes, pixels, out);
-  if (st == JXLR_ENOMEM && *plane) {
+  if (!ctx->cap || ctx->slots.size() == 1) {
+    jxlr_status st = acquire_slot(ctx, need + plane_bytes, pixels, out);
+    if (st != JXLR_ENOMEM || !*plane) return st;
     *plane = false;
-    st = acquire_slot(ctx, need, pixels, out);
+    return acquire_slot(ctx, need, pixels, out);
   }
+  const jxlr_status st = acquire_slot(ctx, need, pixels, out);
+  if (st != JXLR_OK || (*out)->arena_bytes < need + plane_bytes) *plane = false;
   return st;
 }
 
