@@ -957,13 +957,20 @@ extern "C" jxlr_status jxl_recon_submit_jpeg(jxl_recon_ctx* ctx, const jxl_jpeg_
       return fail(JXLR_EINVAL, "submit_jpeg: bad Gaborish side channel");
   }
 
+  // components that come straight from their coefficients in the output
+  // kernel: at full resolution, without the side channel of M.6.3
+  bool direct[3] = {false, false, false};
+  for (int c = 0; c < nc; ++c)
+    direct[c] = static_cast<int>(st->comp[c].h_samp) == hmax &&
+                static_cast<int>(st->comp[c].v_samp) == vmax && !st->comp[c].gab;
+
   size_t need = 0;
   auto add = [&](size_t bytes) { need = align_up(need, 256) + bytes; };
   add(sizeof(unsigned) * kStatusWords);
   for (int c = 0; c < nc; ++c) {
     const size_t nb = static_cast<size_t>(st->comp[c].width_in_blocks) * st->comp[c].height_in_blocks;
     if (!st->on_device) add(nb * 128);
-    add(nb * 256);                                    // sample plane
+    if (!direct[c]) add(nb * 256);                    // sample plane
     if (st->comp[c].gab) add(nb * 256);               // after M.6.3
     if (st->comp[c].cond) {                           // M.6.1.1 results
       for (int k = 0; k < 4; ++k) add(nb * 4);
@@ -1021,7 +1028,7 @@ extern "C" jxlr_status jxl_recon_submit_jpeg(jxl_recon_ctx* ctx, const jxl_jpeg_
         const double eu = u == 0 ? std::sqrt(0.5) : 1.0, ev = v == 0 ? std::sqrt(0.5) : 1.0;
         ia.dq[8 * u + v] = static_cast<float>(k.quant[8 * u + v] * eu * ev / 4.0);
       }
-    ia.plane = cv.take<float>(static_cast<size_t>(bw) * bh * 64);
+    ia.plane = direct[c] ? nullptr : cv.take<float>(static_cast<size_t>(bw) * bh * 64);
     ia.cond = 0;
     std::memset(&ia.c, 0, sizeof(ia.c));
     if (k.cond) {
@@ -1047,9 +1054,8 @@ extern "C" jxlr_status jxl_recon_submit_jpeg(jxl_recon_ctx* ctx, const jxl_jpeg_
       ia.m1 = static_cast<float>(k.quant[0] / 8.0 / std::cos(3.14159265358979323846 / 16.0));
     }
     const float* plane = ia.plane;
-    const bool up = static_cast<int>(k.h_samp) != hmax || static_cast<int>(k.v_samp) != vmax;
-    ca.direct[c] = !up && !k.gab;
-    if (!ca.direct[c]) planes[nplanes++] = ia;
+    ca.direct[c] = direct[c];
+    if (!direct[c]) planes[nplanes++] = ia;
     if (k.gab) {
       JpegGabArgs& ga = gabs[ngabs++];
       ga.src = ia.plane;
