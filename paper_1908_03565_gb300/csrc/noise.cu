@@ -2,17 +2,25 @@
 //
 // Per 256 x 256 group, eight generators run through the three channels
 // row by row, one step per 16-sample segment.  A thread owns one generator
-// for a chunk of 8 rows of one channel: it jumps its state to the chunk's
-// first step with the GF(2) matrices of 2^b steps (the update is linear),
+// for a chunk of 8, 16 or 32 rows of one channel: it jumps its state to the
+// chunk's first step with the GF(2) matrices of 2^b steps (the update is linear),
 // then steps through the chunk, writing samples 2i and 2i+1 of every
 // segment.  The jump replaces up to 12,288 dependent steps per generator by
 // at most 14 matrix-vector products, so the work spreads over all SMs.
 //
 // Bound by the chain of each generator (a step is about 25 dependent integer
-// instructions) and by having enough of them: chunks of 32 rows are 36 CTAs on
-// a 2047x1535 image, fewer than the SMs.  With J.3 and noise the request takes
-// 0.392 ms with chunks of 32 rows, 0.373 with 16, 0.360 with 8 and 0.365 with 4,
-// where the jumps (about 4,600 instructions each) outweigh the steps.
+// instructions), by having enough of them, and where there are, by the jumps
+// (about 4,600 instructions each, once per chunk).  The chunk is the longest
+// that still gives every SM a CTA: 32 rows from 203 groups on (152 SMs), 16 from
+// 102, else 8.  What noise adds to a Gaborish request, us:
+//   image (groups)      8 rows  16 rows  32 rows
+//   1920x1088  (40)         51       55       64
+//   2047x1535  (48)         62       72       89
+//   16384x256  (64)         77       77       81
+//   3001x2003  (96)         79       78       95
+//   4096x4096 (256)        221      197      199
+//   6000x4000 (384)        312      281      275
+//   8192x8192 (1024)       828      741      731
 #include <cuda_runtime.h>
 
 #include "internal.h"
@@ -25,8 +33,6 @@ namespace {
 __constant__ uint64_t c_njump[kNoiseJumpLevels * 256];
 
 constexpr int kGroup = 256;
-constexpr int kChunkRows = 8;
-constexpr int kChunks = kGroup / kChunkRows;
 
 __device__ __forceinline__ uint64_t splitmix64(uint64_t z) {
   z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
@@ -70,7 +76,9 @@ __device__ void gen_jump(uint64_t& s0, uint64_t& s1, int k) {
   }
 }
 
+template <int kRows>
 __global__ void __launch_bounds__(256) k_noise_gen(const __grid_constant__ NoiseGenArgs a) {
+  constexpr int kChunks = kGroup / kRows;
   const long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   const int gi = static_cast<int>(t & 7);
   const long long u = t >> 3;
@@ -81,7 +89,7 @@ __global__ void __launch_bounds__(256) k_noise_gen(const __grid_constant__ Noise
   const int gx = static_cast<int>(g % a.ngx), gy = static_cast<int>(g / a.ngx);
   const int x0 = gx * kGroup, y0 = gy * kGroup;
   const int w = min(kGroup, a.xs - x0), h = min(kGroup, a.ys - y0);
-  const int r0 = q * kChunkRows;
+  const int r0 = q * kRows;
   if (r0 >= h) return;
   const int nseg = (w + 15) >> 4;
   // K.5.2 seeding, generator gi
@@ -93,7 +101,7 @@ __global__ void __launch_bounds__(256) k_noise_gen(const __grid_constant__ Noise
     s1 = splitmix64(s0);
   }
   gen_jump(s0, s1, (c * h + r0) * nseg);
-  const int r1 = min(r0 + kChunkRows, h);
+  const int r1 = min(r0 + kRows, h);
   for (int r = r0; r < r1; ++r) {
     float* row = a.r + c * a.ps + static_cast<size_t>(y0 + r) * a.rs + x0;
     for (int sgi = 0; sgi < nseg; ++sgi) {
@@ -114,8 +122,17 @@ bool upload_noise_constants(const uint64_t* jump) {
 }
 
 int launch_noise_gen(const NoiseGenArgs& a, cudaStream_t s) {
-  const long long threads = static_cast<long long>(a.ngx) * a.ngy * 3 * kChunks * 8;
-  k_noise_gen<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, s>>>(a);
+  static int sms_of[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  int& sms = sms_of[dev & 63];
+  if (sms == 0) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const long long groups = static_cast<long long>(a.ngx) * a.ngy;
+  const auto ctas = [&](int rows) { return (groups * 3 * (kGroup / rows) * 8 + 255) / 256; };
+  const auto grid = [&](int rows) { return static_cast<unsigned>(ctas(rows)); };
+  if (ctas(32) >= sms) k_noise_gen<32><<<grid(32), 256, 0, s>>>(a);
+  else if (ctas(16) >= sms) k_noise_gen<16><<<grid(16), 256, 0, s>>>(a);
+  else k_noise_gen<8><<<grid(8), 256, 0, s>>>(a);
   return 1;
 }
 
