@@ -80,7 +80,6 @@ __global__ void __launch_bounds__(64) k_dc_cell(const __grid_constant__ LfArgs a
   __shared__ uint8_t own[4][4];
   __shared__ uint8_t sv[12][12];          // map of the 3 x 3 cells around this one
   __shared__ float s_up[kLfUpFloats];
-  let_next_start();
   const int tid = threadIdx.x;
   const int cbx = 4 * blockIdx.x, cby = 4 * blockIdx.y;
   const int ox = cbx - 4, oy = cby - 4;
@@ -137,6 +136,12 @@ __global__ void __launch_bounds__(64) k_dc_cell(const __grid_constant__ LfArgs a
     }
     for (int c = 0; c < 3; ++c) dcs[c][ly][lx] = v[c];
   }
+  // from here on the next kernel's blocks may take places: from the start, the
+  // transform kernel's would wait in them, and other streams' kernels for them
+  // (eight requests in flight, 3001x2003 and three 640x480 with F.2 and H in
+  // turn: 103.0 us a request against 101.7; 1920x1088 with and without these
+  // steps 112.6 against 113.2; alone 3001x2003 390 either way)
+  let_next_start();
   if (!a.predict) return;
   __syncthreads();
   // 8 x 8 DC2x2 samples, one per thread, three channels
@@ -184,7 +189,6 @@ __global__ void __launch_bounds__(128) k_lf_cell(const __grid_constant__ LfArgs 
   __shared__ float Us[3][8][8];
   __shared__ float s_inv[kLfInvFloats];
   const int tid = threadIdx.x;
-  let_next_start();
   if (tid < kLfInvFloats) s_inv[tid] = c_lf_inv[tid];
   wait_for_stream();   // k_dc_cell's planes
   const int X0 = 8 * blockIdx.x, Y0 = 8 * blockIdx.y;     // cell origin in DC2x2 samples
@@ -216,6 +220,7 @@ __global__ void __launch_bounds__(128) k_lf_cell(const __grid_constant__ LfArgs 
     Us[c][ly][lx] = (s - t <= wa && wa <= s + t) ? wa : s;
   }
   __syncthreads();
+  let_next_start();   // as in k_dc_cell
 
   for (int i = tid; i < 192; i += 128) {
     const int c = i >> 6, ly = (i >> 3) & 7, lx = i & 7;
