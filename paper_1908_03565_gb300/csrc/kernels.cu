@@ -1375,9 +1375,11 @@ __device__ __forceinline__ void cell_coef_async(const ReconArgs& a, int cxi, int
 // [3][32][32]) and its map entries in the CellMap, put there by the
 // previous cell's call (first: fetched here); with (ncxi, ncyi) >= 0 the
 // next cell's are fetched during this cell's output phase, when T is free.
+// zero: 0, from wait_for_stream() where the kernel was started by launch_after.
 template <bool kTC = false, bool kDc = true, bool kPf = false>
 __device__ __forceinline__ void recon_cell(const ReconArgs& a, int cxi, int cyi, int ncxi = -1,
-                                           int ncyi = -1, bool first = false) {
+                                           int ncyi = -1, bool first = false,
+                                           unsigned zero = 0) {
   __shared__ __align__(16) float S[3][kPR][kRS];
   __shared__ __align__(16) float T[3][kPR][kRS];
   __shared__ CellState cs;
@@ -1432,14 +1434,15 @@ __device__ __forceinline__ void recon_cell(const ReconArgs& a, int cxi, int cyi,
   if (kDc && a.dc1 && tid < 48) {
     const int c = tid >> 4, bx = gbx0 + (tid & 3), by = gby0 + ((tid >> 2) & 3);
     sdc[c][(tid >> 2) & 3][tid & 3] =
-        bx < a.bw && by < a.bh ? a.dc1[c * bpl + static_cast<size_t>(by) * a.bw + bx] : 0.f;
+        bx < a.bw && by < a.bh ? (a.dc1 + zero)[c * bpl + static_cast<size_t>(by) * a.bw + bx] : 0.f;
   }
   if (kDc && a.lfp && tid >= 32) {
     const int i = tid - 32, c = i >> 5, r = (i >> 2) & 7, q = i & 3;
     const int x = 2 * gbx0 + 2 * q, y = 2 * gby0 + r;
     float2 v = make_float2(0.f, 0.f);
     if (x < 2 * a.bw && y < 2 * a.bh)
-      v = *reinterpret_cast<const float2*>(a.lfp + 4 * c * bpl + static_cast<size_t>(y) * (2 * a.bw) + x);
+      v = *reinterpret_cast<const float2*>(a.lfp + zero + 4 * c * bpl +
+                                           static_cast<size_t>(y) * (2 * a.bw) + x);
     *reinterpret_cast<float2*>(&slp[c][r][2 * q]) = v;
   }
   cell_setup(cs, a.vmap, a.acmul, gbx0, gby0, a.bw, a.bh, kTC, a.sigma ? a.sharp : nullptr,
@@ -1671,8 +1674,9 @@ __device__ __forceinline__ void recon_cell(const ReconArgs& a, int cxi, int cyi,
 }
 
 __global__ void __launch_bounds__(128, 7) k_recon(const __grid_constant__ ReconArgs a) {
-  if (a.dc1) wait_for_stream();   // the DC and Annex H kernels, where they come before
-  recon_cell(a, blockIdx.x, blockIdx.y);
+  unsigned zero = 0;
+  if (a.dc1) zero = wait_for_stream();   // the DC and Annex H kernels, where they come before
+  recon_cell(a, blockIdx.x, blockIdx.y, -1, -1, false, zero);
 }
 
 // Persistent form: CTAs take cells cell, cell + gridDim.x, ... (raster

@@ -20,9 +20,11 @@ namespace jxlr {
 // Waits until the kernels before this one in the stream are done and their
 // results visible.  Every thread of a kernel started by launch_after calls it
 // before it reads what they wrote or writes anything (so that a kernel after
-// this one, too, may rely on all of them).  Returns 0: a load whose address has
-// it added cannot be moved before the wait, not even one the compiler takes for
-// a load of constant memory.
+// this one, too, may rely on all of them).  Returns 0, to be added to the
+// addresses of those loads: none of them can be moved before the wait then, not
+// even one that the compiler takes for a load of constant memory (__ldg, or a
+// __restrict__ pointer that the kernel only reads).  Copies by the TMA unit are
+// issued after the wait and need nothing more.
 __device__ __forceinline__ unsigned wait_for_stream() {
   unsigned zero;
   asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero) :: "memory");

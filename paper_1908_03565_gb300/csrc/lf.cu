@@ -190,7 +190,11 @@ __global__ void __launch_bounds__(128) k_lf_cell(const __grid_constant__ LfArgs 
   __shared__ float s_inv[kLfInvFloats];
   const int tid = threadIdx.x;
   if (tid < kLfInvFloats) s_inv[tid] = c_lf_inv[tid];
-  wait_for_stream();   // k_dc_cell's planes
+  const unsigned zero = wait_for_stream();
+  // k_dc_cell's planes
+  const float* const u_in = a.u + zero;
+  const float* const d1_in = a.d1 + zero;
+  const uint8_t* const own_in = a.own + zero;
   const int X0 = 8 * blockIdx.x, Y0 = 8 * blockIdx.y;     // cell origin in DC2x2 samples
   const int pw = 2 * a.bw, ph = 2 * a.bh;
   const int gx0 = X0 & ~63, gy0 = Y0 & ~63;
@@ -201,10 +205,10 @@ __global__ void __launch_bounds__(128) k_lf_cell(const __grid_constant__ LfArgs 
     const int x = X0 - 1 + t % 10, y = Y0 - 1 + t / 10;
     float val;
     if (x >= gx0 && x < gx1 && y >= gy0 && y < gy1) {
-      val = a.u[4 * c * a.bpl + static_cast<size_t>(y) * pw + x];
+      val = u_in[4 * c * a.bpl + static_cast<size_t>(y) * pw + x];
     } else {
       const int bx = mirror1(x >> 1, a.bw), by = mirror1(y >> 1, a.bh);
-      val = a.d1[c * a.bpl + static_cast<size_t>(by) * a.bw + bx];
+      val = d1_in[c * a.bpl + static_cast<size_t>(by) * a.bw + bx];
     }
     U[c][t / 10][t % 10] = val;
   }
@@ -227,7 +231,7 @@ __global__ void __launch_bounds__(128) k_lf_cell(const __grid_constant__ LfArgs 
     const int x = X0 + lx, y = Y0 + ly;
     if (x >= pw || y >= ph) continue;
     const int bx = x >> 1, by = y >> 1;
-    const int o = a.own[static_cast<size_t>(by) * a.bw + bx];
+    const int o = own_in[static_cast<size_t>(by) * a.bw + bx];
     if (o == kNoOwner) continue;
     const int code = o & 15, dx = (o >> 4) & 3, dy = o >> 6;
     const int cx = blocks_w(code), cy = blocks_h(code);
