@@ -83,8 +83,8 @@ typedef struct {
                               several slots a cap admits what the filters' own
                               scratch allows (24 bytes a pixel with the EPF);
                               the 3 bytes a pixel of guide bytes that speed the
-                              EPF up are then kept only in room that a slot's
-                              scratch already has                             */
+                              EPF up are then held where there is room beside
+                              it and given back when a request wants it       */
   int max_slots;           /* requests in flight at once (>= 1); each slot
                               owns one CUDA stream and its scratch arena      */
   int precision;           /* a jxlr_precision                                */

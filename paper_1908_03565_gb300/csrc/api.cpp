@@ -70,6 +70,8 @@ struct Slot {
   bool epf_marked = false;    // marks 5 and 6 were recorded for this request
   char* arena = nullptr;
   size_t arena_bytes = 0;
+  uint8_t* plane = nullptr;       // guide bytes that lie outside the arena
+  size_t plane_bytes = 0;
   unsigned* h_status = nullptr;   // pinned: device status copied back here
   bool busy = false;
   bool timed = false;
@@ -105,6 +107,7 @@ struct jxl_recon_ctx {
   std::atomic<uint64_t> next_ticket{1};
   std::atomic<uint64_t> launches{0};
   size_t bytes = 0;                  // sum of slot arenas
+  size_t planes = 0;                 // sum of slot planes
   std::unordered_map<uint64_t, Timing> timings;
 };
 
@@ -162,7 +165,7 @@ const char* jxl_recon_last_error(const jxl_recon_ctx*) { return g_err.c_str(); }
 
 uint64_t jxl_recon_launch_count(const jxl_recon_ctx* ctx) { return ctx ? ctx->launches.load() : 0; }
 
-size_t jxl_recon_device_bytes(const jxl_recon_ctx* ctx) { return ctx ? ctx->bytes : 0; }
+size_t jxl_recon_device_bytes(const jxl_recon_ctx* ctx) { return ctx ? ctx->bytes + ctx->planes : 0; }
 
 jxlr_status jxl_recon_create(const jxl_recon_config* cfg, jxl_recon_ctx** out) {
   if (!cfg || !out) return fail(JXLR_EINVAL, "create: null argument");
@@ -267,10 +270,9 @@ jxlr_status jxl_recon_destroy(jxl_recon_ctx* ctx) {
   cudaSetDevice(ctx->device);
   for (auto& s : ctx->slots) {
     if (s.stream) cudaStreamSynchronize(s.stream);
-    if (s.arena) {
-      cudaFreeAsync(s.arena, s.stream);
-      cudaStreamSynchronize(s.stream);
-    }
+    if (s.arena) cudaFreeAsync(s.arena, s.stream);
+    if (s.plane) cudaFreeAsync(s.plane, s.stream);
+    if (s.arena || s.plane) cudaStreamSynchronize(s.stream);
     if (s.h_status) cudaFreeHost(s.h_status);
     for (auto& ev : s.ev)
       if (ev) cudaEventDestroy(ev);
@@ -326,6 +328,48 @@ int size_level(uint64_t pixels, int nlevels) {
   return lvl;
 }
 
+// Gives slot s's plane back in the order of `stream`.
+void drop_plane(jxl_recon_ctx* ctx, Slot& s, cudaStream_t stream) {
+  cudaFreeAsync(s.plane, stream);
+  ctx->planes -= s.plane_bytes;
+  s.plane = nullptr;
+  s.plane_bytes = 0;
+}
+
+// Planes give way where slot `best`'s arena is about to grow to `need` bytes and
+// the cap holds the arenas but not the planes too: those of idle slots first, then
+// those of requests in flight, whose end `best`'s stream then waits for (arenas
+// keep their size, so this ends once they have theirs).
+void make_room(jxl_recon_ctx* ctx, Slot* best, size_t need) {
+  const auto over = [&] {
+    return ctx->cap && ctx->bytes - best->arena_bytes + need + ctx->planes > ctx->cap;
+  };
+  for (auto& s : ctx->slots)
+    if (s.plane && !s.busy && over()) drop_plane(ctx, s, s.stream);
+  for (auto& s : ctx->slots)
+    if (s.plane && s.busy && over()) {
+      cudaStreamWaitEvent(best->stream, s.done, 0);
+      drop_plane(ctx, s, best->stream);
+    }
+}
+
+// The slot's plane, of at least `bytes`, or nullptr where it does not fit beside
+// the arenas and the other planes under the cap.
+uint8_t* take_plane(jxl_recon_ctx* ctx, Slot* s, size_t bytes) {
+  if (s->plane_bytes >= bytes) return s->plane;
+  if (s->plane) drop_plane(ctx, *s, s->stream);
+  const size_t sz = align_up(bytes, size_t(1) << 16);
+  if (ctx->cap && ctx->bytes + ctx->planes + sz > ctx->cap) return nullptr;
+  if (cudaMallocAsync(reinterpret_cast<void**>(&s->plane), sz, s->stream) != cudaSuccess) {
+    cudaGetLastError();
+    s->plane = nullptr;
+    return nullptr;
+  }
+  s->plane_bytes = sz;
+  ctx->planes += sz;
+  return s->plane;
+}
+
 // Finds a free slot and makes sure its arena holds `need` bytes within the
 // HBM cap; its stream is the one of the request's size class.  Called with
 // ctx->mu held.
@@ -358,6 +402,7 @@ jxlr_status acquire_slot(jxl_recon_ctx* ctx, size_t need, uint64_t pixels, Slot*
       if (ctx->bytes - best->arena_bytes + need > ctx->cap)
         return fail(JXLR_EBUSY, "not enough HBM under the cap now");
     }
+    make_room(ctx, best, need);
     // stream-ordered: growing an idle slot's arena does not synchronise the
     // device (a plain cudaFree would wait for every request in flight)
     if (best->arena) {
@@ -379,25 +424,27 @@ jxlr_status acquire_slot(jxl_recon_ctx* ctx, size_t need, uint64_t pixels, Slot*
   return JXLR_OK;
 }
 
-// acquire_slot() for a request with the EPF, which can use room for the J.2.2
-// guide bytes behind `need` (*plane: it has it); without, the J.2 kernel forms
-// the bytes from the samples (0.645 instead of 0.602 ms at 4096^2).  With no
-// cap, or with one slot, whose request leaves room for no other, the plane is
-// asked for with the rest and left out where that does not fit.  With several
-// slots under a cap it may cost no request its place, of the later ones
-// neither: the arena is the one that `need` alone asks for, and the plane is
-// used where that has room.
-jxlr_status acquire_epf_slot(jxl_recon_ctx* ctx, size_t need, size_t plane_bytes, uint64_t pixels,
-                             Slot** out, bool* plane) {
-  *plane = plane_bytes != 0;
-  if (!ctx->cap || ctx->slots.size() == 1) {
-    jxlr_status st = acquire_slot(ctx, need + plane_bytes, pixels, out);
-    if (st != JXLR_ENOMEM || !*plane) return st;
-    *plane = false;
+// acquire_slot() for a request with the EPF, and room for its J.2.2 guide bytes
+// (*guide; nullptr: there is none, and the J.2 kernel forms them from the
+// samples, 0.645 instead of 0.602 ms at 4096^2).  With no cap, or with one
+// slot, whose request leaves room for no other, they lie behind `need` in the
+// arena.  With several slots under a cap the arena is the one that `need` alone
+// asks for, and the bytes lie in the slot's plane, which the context takes when
+// there is room beside all arenas and gives back when an arena wants it
+// (make_room): no request loses its place to them, and under a wide cap they all
+// have them (images up to 8192^2 served in eight slots under 40 GB at a tenth of
+// the capacity: p99 1.82 ms where arenas alone had room for them, 1.69 so).
+jxlr_status acquire_epf_slot(jxl_recon_ctx* ctx, size_t need, size_t guide_bytes, uint64_t pixels,
+                             Slot** out, uint8_t** guide) {
+  *guide = nullptr;
+  if (guide_bytes && (!ctx->cap || ctx->slots.size() == 1)) {
+    const jxlr_status st = acquire_slot(ctx, need + guide_bytes, pixels, out);
+    if (st == JXLR_OK) *guide = reinterpret_cast<uint8_t*>((*out)->arena + need);
+    if (st != JXLR_ENOMEM) return st;
     return acquire_slot(ctx, need, pixels, out);
   }
   const jxlr_status st = acquire_slot(ctx, need, pixels, out);
-  if (st != JXLR_OK || (*out)->arena_bytes < need + plane_bytes) *plane = false;
+  if (st == JXLR_OK && guide_bytes) *guide = take_plane(ctx, *out, guide_bytes);
   return st;
 }
 
@@ -568,15 +615,15 @@ extern "C" jxlr_status jxl_recon_submit(jxl_recon_ctx* ctx, const jxl_recon_coef
   const size_t out_bytes = out->row_stride_bytes * (ys - 1) + px_bytes * xs;
   if (!out->on_device) add(out_bytes);
   need = align_up(need, 256);
-  const size_t plane_bytes = fp->epf ? align_up(3 * 64 * nblk, 256) : 0;   // J.2.2 guide bytes
+  const size_t guide_bytes = fp->epf ? align_up(3 * 64 * nblk, 256) : 0;   // J.2.2 guide bytes
 
   std::lock_guard<std::mutex> lock(ctx->mu);
   CK(cudaSetDevice(ctx->device));
   Slot* slot = nullptr;
-  bool plane = false;
-  jxlr_status st = acquire_epf_slot(ctx, need, plane_bytes,
+  uint8_t* guide = nullptr;
+  jxlr_status st = acquire_epf_slot(ctx, need, guide_bytes,
                                     static_cast<uint64_t>(xs) * static_cast<uint64_t>(ys), &slot,
-                                    &plane);
+                                    &guide);
   if (st != JXLR_OK) return st;
   slot->timed = ctx->timing;
   slot->epf_marked = false;
@@ -694,7 +741,7 @@ extern "C" jxlr_status jxl_recon_submit(jxl_recon_ctx* ctx, const jxl_recon_coef
       sink.pass = eo;
       sink.prs = wp;
       sink.pps = static_cast<size_t>(wp) * hp;
-      if (plane) sink.guide = reinterpret_cast<uint8_t*>(slot->arena + need);
+      sink.guide = guide;
     }
     ra.write_xyb = 1;
     ra.xyb = xyb;
@@ -760,14 +807,14 @@ extern "C" jxlr_status jxl_recon_submit_xyb(jxl_recon_ctx* ctx, const float* xyb
     need += align_up(sizeof(int) * static_cast<size_t>(bw) * bh, 256);
   }
   if (fp->noise) need += align_up(sizeof(float) * 3 * static_cast<size_t>(xs) * ys, 256);
-  const size_t plane_bytes = fp->epf ? align_up(size_t(3) * 64 * bw * bh, 256) : 0;
+  const size_t guide_bytes = fp->epf ? align_up(size_t(3) * 64 * bw * bh, 256) : 0;
   std::lock_guard<std::mutex> lock(ctx->mu);
   CK(cudaSetDevice(ctx->device));
   Slot* slot = nullptr;
-  bool plane = false;
-  jxlr_status st = acquire_epf_slot(ctx, need, plane_bytes,
+  uint8_t* guide = nullptr;
+  jxlr_status st = acquire_epf_slot(ctx, need, guide_bytes,
                                     static_cast<uint64_t>(xs) * static_cast<uint64_t>(ys), &slot,
-                                    &plane);
+                                    &guide);
   if (st != JXLR_OK) return st;
   slot->timed = ctx->timing;
   slot->epf_marked = false;
@@ -795,7 +842,7 @@ extern "C" jxlr_status jxl_recon_submit_xyb(jxl_recon_ctx* ctx, const float* xyb
     sink.pass = eo;
     sink.prs = static_cast<size_t>(8) * bw;
     sink.pps = static_cast<size_t>(64) * bw * bh;
-    if (plane) sink.guide = reinterpret_cast<uint8_t*>(slot->arena + need);
+    sink.guide = guide;
     SigmaArgs sa;
     std::memset(&sa, 0, sizeof(sa));
     sa.xyb = xyb;

@@ -1,6 +1,7 @@
 """Requests in flight together under an HBM cap: the guide bytes that J.2 can
-use cost none of them its place.  What the context admits and the bytes it
-holds are those of the filters' own scratch, computed here."""
+use cost none of them its place.  What the context admits is what the
+filters' own scratch, computed here, allows; it holds that and, as far as the cap
+leaves room, guide bytes."""
 import numpy as np
 import pytest
 
@@ -91,12 +92,15 @@ def test_two_at_once(gpu_lib, kind, extra):
         w = Work(torch, ctx, 1024, 1024, kind)
     with binding.Context(device=0, max_slots=2, hbm_cap_bytes=up(w.need, MiB) + w.need + extra) as ctx:
         got = [w.submit(ctx)]
+        assert ctx.device_bytes() == up(w.need, MiB) + 3 * MiB     # with its guide bytes
         if extra < 0:
             with pytest.raises(binding.JxlrError) as e:
                 w.submit(ctx)
             assert e.value.status == binding.JXLR_EBUSY
         else:
             got.append(w.submit(ctx))
+            # the first one's stay where the second one's scratch leaves room
+            assert ctx.device_bytes() == 2 * up(w.need, MiB) + (3 * MiB if extra == 5 * MiB else 0)
         for out, t in got:
             ctx.poll(t)
             assert w.right(out)
@@ -110,7 +114,7 @@ def test_any_order(gpu_lib):
                  for xs, ys in [(131, 77), (520, 392), (768, 512), (1024, 1024)]
                  for kind in ("gab", "epf", "xyb")]
     model = Slots(4, 37 * MiB)
-    flight, refused = [], 0
+    flight, refused, kept = [], 0, 0
     with binding.Context(device=0, max_slots=4, hbm_cap_bytes=model.cap) as ctx:
         for _ in range(240):
             if flight and rng.random() < 0.4:
@@ -128,8 +132,10 @@ def test_any_order(gpu_lib):
             except binding.JxlrError as e:
                 assert e.status == want
                 refused += not all(model.busy)
-            assert ctx.device_bytes() == sum(model.arena)
+            assert 0 <= ctx.device_bytes() - sum(model.arena) <= max(0, model.cap - sum(model.arena)) + MiB
+            kept += ctx.device_bytes() > sum(model.arena)
         for w, s, out, t in flight:
             ctx.poll(t)
             assert w.right(out)
     assert refused > 5    # refusals by the cap, not for want of a slot
+    assert kept > 5       # times with guide bytes beside the scratch
