@@ -32,17 +32,17 @@ SEED = 2000
 # 3 float32)
 IN_BPP = 6.0 + 1 / 64 + 4 / 64 + 1 / 64 + 8 / 4096
 OUT_BPP = 12.0
-# algorithmic lane operations of the J.2 kernel, a lower bound that holds on
-# any data: per pixel it filters (those of the 8x8 blocks with sigma >= 16;
-# the others pass through), per offset the patch SAD on packed guide bytes
-# with separable 3x4 sums (absdiff 1, channel sum 1, horizontal and vertical
-# sliding sums 4) and the J.2.4 cut-off test (multiply-add 1, compare 1)
-# (x 56), the J.2.5 accumulation of the centre sample, whose weight is always
-# 1 (4), normalisation 4; per pixel of the image, the guide 17.  The
-# accumulation of the other samples whose weights pass the cut-off (4 per
-# such pixel and offset) depends on the data and is not counted.
-EPF_OPS_PER_FILTERED_PX = 56 * 8 + 4 + 4
-GUIDE_OPS_PER_PX = 17
+# lane operations that the form of the J.2 kernel (planar guide words) needs at
+# the least, on any data: per pixel it filters (those of the 8x8 blocks with
+# sigma >= 16; the others pass through), per offset one patch row of the three
+# channels (a byte-SAD takes 4 columns: 3; its other two rows are its
+# neighbours'), the sum of the three rows 1 and the minimum for the J.2.4
+# cut-off test 1 (x 56), the J.2.5 accumulation of the centre sample, whose
+# weight is always 1 (4), normalisation 4.  Another form may need fewer (one
+# SAD per pixel needed 456).  The accumulation of the other samples whose
+# weights pass the cut-off (4 per such pixel and offset) depends on the data and
+# is not counted; the guide bytes are the transform kernel's.
+EPF_OPS_PER_FILTERED_PX = 56 * 5 + 4 + 4
 # DRAM bytes (read + write) of one k_epf_work launch, from an ncu capture of
 # the current kernel on the same statistics at 4096x2048 (50,730 listed
 # blocks): 102,867,200 + 19,798,784; scaled to a launch by its pixels.  Set to
@@ -464,7 +464,7 @@ def epf_active_leg(binding, torch, steps, alu_peak):
         epf = np.array([ctx.epf_stats(t) for t in tickets])
     epf_ms, blocks = float(epf[:, 0].mean()), int(epf[-1, 1])
     nblk = ((XS + 7) // 8) * ((YS + 7) // 8)
-    ops = (EPF_OPS_PER_FILTERED_PX * 64 * blocks + GUIDE_OPS_PER_PX * XS * YS) / (epf_ms * 1e-3) / 1e12
+    ops = EPF_OPS_PER_FILTERED_PX * 64 * blocks / (epf_ms * 1e-3) / 1e12
     return {"ms_per_step": round(ms, 4), "mpx_s": round(XS * YS / ms / 1e3, 1),
             "epf_ms": round(epf_ms, 4), "filtered_frac": round(blocks / nblk, 4),
             "epf_alu_frac": round(ops / alu_peak, 4),
@@ -792,8 +792,7 @@ def main():
     sm_mhz = peaks.get("sm_max_mhz", 2070.0)
     alu_peak = sm_count * 128 * sm_mhz * 1e6 / 1e12      # T lane-ops/s
     nblk = ((XS + 7) // 8) * ((YS + 7) // 8)
-    achieved_alu = (EPF_OPS_PER_FILTERED_PX * 64 * epf_blocks + GUIDE_OPS_PER_PX * px) / \
-        (epf_ms * 1e-3) / 1e12
+    achieved_alu = EPF_OPS_PER_FILTERED_PX * 64 * epf_blocks / (epf_ms * 1e-3) / 1e12
     recon_gbs = px * (IN_BPP + 12.0 + 4 / 64) / (recon_ms * 1e-3) / 1e9  # reads coefs, writes XYB
     epf_traffic = (None if EPF_WORK_DRAM_BYTES_4096x2048 is None else
                    int(round(EPF_WORK_DRAM_BYTES_4096x2048 * px / (4096 * 2048))))

@@ -263,8 +263,9 @@ jxlr_status jxl_recon_poll(jxl_recon_ctx* ctx, uint64_t ticket, int64_t timeout_
                            double* latency_ms);
 
 /* Device time of each stage of a finished request, in ms, when the
- * context was created with timing = 1: ms[0] validation (0: the
- * transform kernel checks device maps), ms[1] dequantisation + transforms, ms[2] filters + colour, ms[3] host<->device
+ * context was created with timing = 1: ms[0] validation (about 0 where the
+ * transform kernel checks the device map, within ms[1]), ms[1]
+ * dequantisation + transforms, ms[2] filters + colour, ms[3] host<->device
  * copies.  Call after jxl_recon_poll() returned JXLR_OK for the ticket;
  * the values stay until the next completed request of that slot. */
 jxlr_status jxl_recon_stage_ms(jxl_recon_ctx* ctx, uint64_t ticket, float ms[4]);

@@ -1,7 +1,8 @@
 // CUDA kernels of VarDCT pixel reconstruction for sm_103a (GB300).
 //
 //   k_validate  C.5.4: the DctSelect map must tile the image with naturally
-//               aligned, in-bounds varblocks.
+//               aligned, in-bounds varblocks (submit_xyb and batches; for a
+//               submit's device map k_recon checks each cell).
 //   k_recon     one 32x32 cell per CTA (varblocks are naturally aligned and
 //               at most 32x32, so each lies inside one cell):
 //               F.2/F.3 dequantisation with 128-bit int16 loads, G chroma
@@ -23,7 +24,7 @@
 // draft's transforms is folded into the dequantisation tables and the LLF
 // maps on the host.  The 1-D sums use the even/odd split
 // x[n] = E[n] + O[n], x[N-1-n] = E[n] - O[n] recursively, with the odd-part
-// cosine matrices in constant memory.
+// cosines as immediate operands (odd_cos).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
@@ -1016,7 +1017,7 @@ __device__ void cell_setup(CellState& cs, const uint8_t* __restrict__ vmap,
     if (tid < 16 && code < kNumCodes) {
       w8 = 1 << lg_w8(code);
       h8 = 1 << lg_h8(code);
-      // ill-formed placements are reported by k_validate; skip them here
+      // ill-formed placements are skipped (and reported, below or by k_validate)
       valid = !(bx % w8 || by % h8 || bx + w8 > 4 || by + h8 > 4 || gbx0 + bx + w8 > bw ||
                 gby0 + by + h8 > bh);
       ri = tc && tc_shape(code) ? 0 : row_items(code);

@@ -4,12 +4,14 @@
 // A plain launch starts after the last block of the kernel before it has ended
 // and its writes are flushed, 3-4 us in which a request's next kernel does
 // nothing; launched this way its blocks are already in place.  Measured (one
-// request at a time, J.2 and Gaborish / colour kernels launched this way): 48x40
-// u8 73 -> 64 us, 1920x1088 u8 125 -> 119, 4096x4096 f32 530 -> 527, 8192x8192
-// the same; without let_next_start in the transform kernel 4096x4096 is 2-4 us
-// slower.  The DC kernels (F.2, H) and the transform kernel behind them:
-// 3001x2003 photograph 400 -> 393 us.  The JPEG1 output kernel behind its chroma planes gained nothing
-// (4096x4096 113 us either way).
+// request at a time, host's wait included, both sides in one session; J.2 and
+// Gaborish / colour kernels launched this way): 48x40 u8 73 -> 64 us, 1920x1088
+// u8 125 -> 119, 4096x4096 f32 530 -> 527, 8192x8192 the same; without
+// let_next_start in the transform kernel 4096x4096 is 2-4 us slower.  The DC
+// kernels (F.2, H) and the transform kernel behind them: 3001x2003 photograph
+// 400 -> 393 us.  With several requests in flight a kernel lets the next one in
+// only after its main work (k_dc_cell).  The JPEG1 output kernel behind its
+// chroma planes gained nothing (4096x4096 113 us either way): a plain launch.
 #ifndef JXLR_LAUNCH_H_
 #define JXLR_LAUNCH_H_
 
